@@ -318,7 +318,8 @@ void ns_free(ns_ctx *c) {
     if (c->graph) cudaGraphExecDestroy(c->graph);
     for (cudaEvent_t e : c->ev)
         if (e) cudaEventDestroy(e);
-    void *bufs[] = {c->d_re, c->d_im, c->d_psd, c->basis64, c->f64, c->prefix, c->w64, c->X.basis32,
+    void *bufs[] = {c->d_re, c->d_im, c->d_psd, c->basis64, c->f64, c->prefix, c->w64, c->fx.b, c->fx.f, c->fx.w, c->fx.scale,
+                    c->fx.sc, c->fx.wmax, c->X.basis32,
                     c->X.f32, c->X.w32, c->X.tb0, c->X.tb1, c->X.tbk, c->X.fc, c->X.wt, c->live_u, c->live_logl, c->order, c->chol, c->dead_u,
                     c->dead_logl, c->dead_logw, c->dead_nlive, c->state, c->scratch, c->fin_u,
                     c->fin_logl, c->fin_logw, c->fin_nlive, c->res, c->rb_J, c->rb_nedge, c->rb_fid,
@@ -464,6 +465,45 @@ static int alloc_mixed(ns_ctx *c) {
     return NS_OK;
 }
 
+// FP64 form: the split tables (not for relative binning, whose likelihood reads
+// the coarse bins), and the binary exponents that bring the basis functions and
+// the frequency below one: each is monotone on the grid but f^(1/3) ln f, whose
+// minimum is -3/e at f = e^-3.
+static int alloc_fx(ns_ctx *c, int coarse_bins) {
+    const Model &M = c->M;
+    if (M.model != M_GW || c->precision != NS_FP64 || coarse_bins > 0) return NS_OK;
+    const size_t N = M.N, nd = M.n_det;
+    int rc;
+    if ((rc = dalloc(&c->w64, nd * N)) || (rc = dalloc(&c->fx.b, NB / 2 * N)) || (rc = dalloc(&c->fx.f, N)) ||
+        (rc = dalloc(&c->fx.w, nd * N)) || (rc = dalloc(&c->fx.scale, nd)) || (rc = dalloc(&c->fx.wmax, nd)) ||
+        (rc = dalloc(&c->fx.sc, gwns::FX_SC)))
+        return rc;
+    c->fx.n = M.N;
+    double mx[NB + 1] = {};
+    for (const double f : {M.f0, M.f0 + (double)(M.N - 1) * M.df}) {
+        const double r = std::cbrt(f), l = std::log(f);
+        const double B[NB + 1] = {1.0 / (f * r * r), 1.0 / f, 1.0 / (r * r), 1.0 / r, l, r, r * l, r * r, f};
+        for (int m = 0; m <= NB; m++) mx[m] = std::max(mx[m], std::fabs(B[m]));
+    }
+    mx[6] = std::max(mx[6], 1.2);
+    for (int m = 0; m <= NB; m++) c->T.fxe[m] = std::ilogb(std::max(mx[m] * (1.0 + 1e-12), 1e-300)) + 1;
+    c->T.fxb = c->fx.b;
+    c->T.fxf = c->fx.f;
+    c->T.fxw = c->fx.w;
+    c->T.fxs = c->fx.scale;
+    c->T.fxsc = c->fx.sc;
+    c->T.fxn = c->fx.n;
+    return NS_OK;
+}
+
+// Tables of the current data, on the context's stream.
+static cudaError_t build_tables(ns_ctx *c) {
+    cudaError_t e = launch_build_tables(c->M, c->d_re, c->d_im, c->d_psd, c->basis64, c->f64, c->w64, c->prefix, c->X,
+                                        c->stream);
+    if (e == cudaSuccess && c->fx.b) e = launch_build_fx(c->M, c->T, c->w64, c->fx, c->stream);
+    return e;
+}
+
 int ns_init(ns_ctx **out, const ns_prior *prior, const ns_data *data, const ns_psd *psd,
             const ns_grid *grid, const ns_options *o) {
     if (!out) return NS_ERR_INVALID_ARG;
@@ -569,7 +609,7 @@ int ns_init(ns_ctx **out, const ns_prior *prior, const ns_data *data, const ns_p
     const size_t N = M.N, nd = M.n_det, nn = nd * N;
     if ((rc = dalloc(&c->d_re, nn)) || (rc = dalloc(&c->d_im, nn)) || (rc = dalloc(&c->d_psd, nn)) ||
         (rc = dalloc(&c->basis64, NB * N)) || (rc = dalloc(&c->f64, N)) || (rc = dalloc(&c->prefix, nn)) ||
-        (rc = dalloc(&c->w64, nn)) || (rc = alloc_mixed(c)) || (rc = dalloc(&c->live_u, (size_t)c->n * c->d)) ||
+        (rc = alloc_fx(c, grid ? grid->coarse_bins : 0)) || (rc = alloc_mixed(c)) || (rc = dalloc(&c->live_u, (size_t)c->n * c->d)) ||
         (rc = dalloc(&c->live_logl, c->n)) || (rc = dalloc(&c->order, c->n)) ||
         (rc = dalloc(&c->chol, (size_t)NS_MAX_DIM * NS_MAX_DIM)) || (rc = dalloc(&c->state, 1)) ||
         (rc = dalloc(&c->fin_u, (size_t)c->n * c->d)) || (rc = dalloc(&c->fin_logl, c->n)) ||
@@ -618,18 +658,15 @@ int ns_init(ns_ctx **out, const ns_prior *prior, const ns_data *data, const ns_p
             e = cudaMemsetAsync(c->d_re, 0, nn * sizeof(double), c->stream);
             if (e == cudaSuccess) e = cudaMemsetAsync(c->d_im, 0, nn * sizeof(double), c->stream);
         }
-        if (e == cudaSuccess)
-            e = launch_build_tables(M, c->d_re, c->d_im, c->d_psd, c->basis64, c->f64, c->w64, c->prefix,
-                                    c->X, c->stream);
+        c->T.basis64 = c->basis64;
+        c->T.f64 = c->f64;
+        if (e == cudaSuccess) e = build_tables(c);
     }
     if (e != cudaSuccess) { ns_free(c); return cuda_fail(e); }
     if (M.model == M_GW && grid->coarse_bins > 0) {
         c->rb_B = grid->coarse_bins;
         for (int p = 0; p < NS_NPARAM; p++) c->rb_theta[p] = grid->theta_fid[p];
     }
-    c->T.basis64 = c->basis64;
-    c->T.f64 = c->f64;
-    c->T.w64 = c->w64;
     c->T.prefix = c->prefix;
     c->T.basis32 = c->X.basis32;
     c->T.f32 = c->X.f32;
@@ -665,8 +702,7 @@ int ns_set_data(ns_ctx *c, const double *re, const double *im) {
     const size_t nn = (size_t)c->M.n_det * c->M.N;
     CK(cudaMemcpyAsync(c->d_re, re, nn * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->d_im, im, nn * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    CK(launch_build_tables(c->M, c->d_re, c->d_im, c->d_psd, c->basis64, c->f64, c->w64, c->prefix, c->X,
-                           c->stream));
+    CK(build_tables(c));
     int rc;
     if (c->rb_B > 0 && (rc = build_rb(c))) return rc;
     rc = eval_points(c, c->live_u, 0, c->n, c->live_logl);

@@ -33,7 +33,8 @@ struct ns_ctx {
     // device buffers
     double *d_re = nullptr, *d_im = nullptr, *d_psd = nullptr;
     double *basis64 = nullptr, *f64 = nullptr, *prefix = nullptr;
-    double2 *w64 = nullptr;
+    double2 *w64 = nullptr;          // FP64 form only
+    gwns::FxTables fx = {};          // FP64 form's split tables
     MixedTables X = {};   // mixed-form tables (per-bin or tiled)
     double *live_u = nullptr, *live_logl = nullptr;
     int *order = nullptr;

@@ -18,6 +18,7 @@
 #include <stdint.h>
 
 #include "gwns_df.cuh"
+#include "gwns_fx.cuh"
 #include "gwns_tables.cuh"
 
 namespace gwns {
@@ -88,7 +89,14 @@ struct RBTables {
 struct Tables {
     const double *basis64;   // [NB][N]   B_m(f_j)
     const double *f64;       // [N]       f_j
-    const double2 *w64;      // [n_det][N] weighted data
+    // FP64 form (gwns_fx.cuh)
+    const int4 *fxb;         // [NB/2][fxn] basis functions 2i and 2i+1 as fx2 pairs
+    const int2 *fxf;         // [fxn]     f_j as fx2
+    const float4 *fxw;       // [n_det][fxn] weighted data / fxs[d], double-float (re h, re l, im h, im l)
+    const double *fxs;       // [n_det]   power-of-two scale of the weighted data
+    const float4 *fxsc;      // [FX_SC]   cos and sin of k 2 pi/1024, double-float
+    int fxn;                 // rows of fxb, fxf and fxw
+    int fxe[NB + 1];         // binary exponents of the basis functions' and the frequency's scale
     const double *prefix;    // [n_det][N] P_d(j)
     // mixed form, per bin (Model::tlg == 0)
     const float2 *basis32;   // [NB][N]   B_m(f_j) as (hi, lo) floats
@@ -109,11 +117,11 @@ struct Tables {
 struct Coef {
     double a[NB];          // phase coefficients [rad per basis unit]
     double c0;             // constant phase [rad]
+    double c0u;            // the same, not reduced by turns
     double tau[MAXDET];    // t_c + dt_d [s]
     double gre[MAXDET], gim[MAXDET];   // G_d = A conj(Q_d)
     double hh;             // sum_d <h_d|h_d>
     double toy;            // toy model log L
-    double rot_re[MAXDET], rot_im[MAXDET];   // exp(2 pi i rot_stride df tau_d) (FP64 loop)
     double fisco;          // f_ISCO [Hz]
     double amp;            // Newtonian amplitude factor A
     int jcut;              // last bin with f_j <= f_ISCO (-1: none)
@@ -291,11 +299,9 @@ __device__ const dfl PN_POLY_X[NB * 4] = {GWNS_PN_POLY(DFC)};
 // log, one exp, one sincos), and the detector terms run on sub-lanes
 // 0 .. n_det-1. The distance enters only through ln D_L, so a uniform-in-volume
 // distance needs no cube root. u0 + g*ustride: point g's unit-cube coordinates;
-// out0[g]: its coefficients. rot_stride > 0 also stores, per detector,
-// exp(2 pi i rot_stride df tau_d), the rotation between bins rot_stride apart
-// used by the FP64 bin loop. GW model only; all 32 lanes must call.
+// out0[g]: its coefficients. GW model only; all 32 lanes must call.
 __device__ inline void point_coef_group(const Model &M, const Tables &T, const double *u0, int ustride,
-                                        Coef *out0, int count, int rot_stride, int half = 0) {
+                                        Coef *out0, int count, int half = 0) {
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, g = lane >> 3, sl = lane & 7;
     const bool writer = g < count;
@@ -338,24 +344,31 @@ __device__ inline void point_coef_group(const Model &M, const Tables &T, const d
         const double delta = (1.0 - q) * r1q;           // (m1 - m2)/M, m1 >= m2
         const double chis = 0.5 * (th[P_CHI1] + th[P_CHI2]);
         const double chia = 0.5 * (th[P_CHI1] - th[P_CHI2]);
-        const double tmc = th[P_MC] * TSUN;
-        // packed log: sub-lane 0 ln(eta), 1 ln(T_Mc), others ln(D_L) (or of D_L^3)
-        const double lg = log_tab(sl == 0 ? eta : (sl == 1 ? tmc : dl_arg));
+        // The logarithms are taken of the mass in solar units and the powers of
+        // T_sun (and the amplitude's constants) multiplied in after the exponential:
+        // the exponents stay below 12, and with them the rounding that the
+        // exponential turns into a relative error (with the constants inside, up to
+        // -60; relative error of log L against 80-bit arithmetic over prior draws,
+        // 64,897 / 519,169 bins: 3.2e-15 / 1.1e-11 -> 1.7e-15 / 5.5e-12).
+        // packed log: sub-lane 0 ln(eta), 1 ln(Mc), others ln(D_L) (or of D_L^3)
+        const double lg = log_tab(sl == 0 ? eta : (sl == 1 ? th[P_MC] : dl_arg));
         const double ln_eta = __shfl_sync(FULL, lg, 0, 8);
-        const double ln_tmc = __shfl_sync(FULL, lg, 1, 8);
+        const double ln_mc = __shfl_sync(FULL, lg, 1, 8);
         const double ln_dlx = __shfl_sync(FULL, lg, 2, 8);
         const double ln_dl = dl_vol ? ln_dlx * (1.0 / 3.0) : ln_dlx;
-        // ln(pi T_M) with T_M = T_Mc eta^(-3/5); a = (pi T_M)^(1/3), v = a f^(1/3)
-        const double ln_x = 1.1447298858494002 + ln_tmc - 0.6 * ln_eta;
-        const double ln_a = ln_x * (1.0 / 3.0);
+        // x = M / M_sun = Mc eta^(-3/5); a = (pi T_sun x)^(1/3), v = a f^(1/3)
+        const double ln_x = ln_mc - 0.6 * ln_eta;
+        const double ln_x3 = ln_x * (1.0 / 3.0);
+        const double ln_a = ln_x3 - 3.6921189058862547;                  // + ln(pi T_sun)/3
         // packed exp: 0 a, 1 1/a, 2 1/(pi T_M), 3 K = 3/(128 eta),
         // others A = sqrt(5/24) pi^(-2/3) c T_Mc^(5/6) / D_L (D_L in Mpc)
-        const double ex_arg = sl == 0 ? ln_a
-                            : sl == 1 ? -ln_a
+        const double ex_arg = sl == 0 ? ln_x3
+                            : sl == 1 ? -ln_x3
                             : sl == 2 ? -ln_x
-                            : sl == 3 ? -3.7534179752515073 - ln_eta
-                            : -33.81250354619071 + (5.0 / 6.0) * ln_tmc - ln_dl;
-        const double ex = exp_tab(ex_arg);
+                            : sl == 3 ? -ln_eta
+                            : (5.0 / 6.0) * ln_mc - ln_dl;
+        const double ex_c = sl == 0 ? 0.02491914473975832 : sl == 1 ? 40.12978817866518 : sl == 2 ? 64625.006840429545 : sl == 3 ? 3.0 / 128.0 : 7.806521525937891e-20;
+        const double ex = exp_tab(ex_arg) * ex_c;
         const double a = __shfl_sync(FULL, ex, 0, 8);
         const double ia = __shfl_sync(FULL, ex, 1, 8);
         const double inv_pitm = __shfl_sync(FULL, ex, 2, 8);
@@ -395,6 +408,7 @@ __device__ inline void point_coef_group(const Model &M, const Tables &T, const d
             const double phi5 = pi * (38645.0 / 756.0 - 65.0 / 9.0 * eta) - gamma;
             const double c0 = -th[P_PHIC] - 0.25 * pi + K * phi5 * (1.0 + 3.0 * 0.8958797346140275 + 3.0 * ln_a);
             out->c0 = c0 - TWO_PI_D * rint(c0 * INV_TWO_PI_D);
+            out->c0u = c0;
             out->jcut = jcut;
             out->fisco = inv_pitm * 0.06804138174397717;
             out->amp = amp;
@@ -408,7 +422,7 @@ __device__ inline void point_coef_group(const Model &M, const Tables &T, const d
     sincos_bf(sl == 0 ? th[P_RA] : th[P_PSI], sn, cs);
     const double sa = __shfl_sync(FULL, sn, 0, 8), ca = __shfl_sync(FULL, cs, 0, 8);
     const double sp = __shfl_sync(FULL, sn, 1, 8), cp = __shfl_sync(FULL, cs, 1, 8);
-    double hh_part = 0.0, tau = 0.0;
+    double hh_part = 0.0;
     if (sl < M.n_det) {
         const int dd = sl;
         double fp, fc, dt;
@@ -433,20 +447,14 @@ __device__ inline void point_coef_group(const Model &M, const Tables &T, const d
         }
         const double qre = fp * 0.5 * (1.0 + ci * ci);
         const double qim = -fc * ci;
-        tau = th[P_TC] + dt;
         if (writer) {
-            out->tau[dd] = tau;
+            out->tau[dd] = th[P_TC] + dt;
             // half 2 leaves the amplitude to point_coef_join
             out->gre[dd] = half == 2 ? qre : amp * qre;
             out->gim[dd] = half == 2 ? -qim : -amp * qim;
         }
         if (half == 0 && jcut >= 0)
             hh_part = amp * amp * (qre * qre + qim * qim) * T.prefix[(size_t)dd * M.N + jcut];
-    }
-    if (rot_stride > 0) {
-        double rs, rc;
-        sincos(TWO_PI_D * ((double)rot_stride * M.df) * tau, &rs, &rc);
-        if (sl < M.n_det && writer) { out->rot_re[sl] = rc; out->rot_im[sl] = rs; }
     }
     if (half == 2) return;
 #pragma unroll
@@ -475,8 +483,7 @@ __device__ __forceinline__ void point_coef_join(const Model &M, const Tables &T,
 }
 
 // Coefficients of one point by one warp (toy model, or GW via lane group 0).
-__device__ inline void point_coef_warp(const Model &M, const Tables &T, const double *u, Coef *out,
-                                       int rot_stride = 0) {
+__device__ inline void point_coef_warp(const Model &M, const Tables &T, const double *u, Coef *out) {
     const int lane = threadIdx.x & 31;
     if (M.model == M_TOY) {
         // log N(x; 0, Sigma) with Sigma_ij = rho^|i-j|: the inverse is tridiagonal,
@@ -498,7 +505,7 @@ __device__ inline void point_coef_warp(const Model &M, const Tables &T, const do
         }
         return;
     }
-    point_coef_group(M, T, u, 0, out, 1, rot_stride);
+    point_coef_group(M, T, u, 0, out, 1);
 }
 
 // Split a double into (hi, lo) floats.
@@ -779,67 +786,86 @@ __device__ __forceinline__ void sincos_bf(double x, double &s, double &c) {
     c = ((q + 1) & 2) ? -b : b;
 }
 
-// FP64: Psi_j from the basis (FP64 FMAs), exp(i Psi_j) by sincos, the detector
-// factor exp(2 pi i f_j tau_d) by a rotation recurrence along the thread's bins
-// (f advances by stride*df per step).
-// With PRE_ROT the coefficients carry the rotation for a stride of 32 bins;
-// the stride here is 32 << rot_sq (the rotation squared rot_sq times).
-template <int NDET, bool PRE_ROT = false>
-__device__ __forceinline__ void bins_fp64(const Tables &T, int N, double f0, double df, const Coef &c,
-                                          int tid, int stride, double zr[NDET], double zi[NDET],
-                                          int rot_sq = 0) {
-    double a[NB];
+// FP64 form: the coefficients of up to four points as fixed-point integers on
+// one scale per point (gwns_fx.cuh): lane group g (8 lanes) takes point g, its
+// sub-lane m basis coefficient m, then detector m's delay and (sub-lane 0) the
+// constant phase. Integer instructions only. All 32 lanes must call.
+__device__ inline void coef_to_fx_group(const Tables &T, int n_det, const Coef *c0, FxPoint *out0, int count) {
+    const int lane = threadIdx.x & 31, g = lane >> 3, sl = lane & 7;
+    const bool writer = g < count;
+    const Coef &c = c0[writer ? g : 0];
+    FxPoint &o = out0[writer ? g : 0];
+    int bad = 0;
+    uint64_t ma, mt, mc;
+    const bool det = sl < n_det;
+    const double a = c.a[sl], tau = c.tau[det ? sl : 0], ph = c.c0u;
+    const int ea = fx_mantissa<true>(a, &ma, &bad) + T.fxe[sl];
+    const int et = fx_mantissa<false>(tau, &mt, &bad) + T.fxe[NB];
+    const int ec = fx_mantissa<true>(ph, &mc, &bad);
+    // the point's scale 2^E: above every term's largest value on the grid
+    int E = max(max(max(ea, et), ec) + 64, 0);
+#pragma unroll
+    for (int w = 4; w > 0; w >>= 1) {
+        E = max(E, __shfl_xor_sync(0xffffffffu, E, w, 8));
+        bad |= __shfl_xor_sync(0xffffffffu, bad, w, 8);
+    }
+    if (!writer) return;
+    o.a[sl] = fx_split(fx_scaled(ma, E - (ea + 64) + 6, a));
+    if (det) o.t[sl] = fx_split(fx_scaled(mt, E - (et + 64) + 6, tau));
+    if (sl == 0) {
+        o.c0 = fx_scaled(mc, E - (ec + 64) + 7, ph);
+        o.sh = E + 7;
+        o.bad = bad;
+    }
+}
+
+// The FX_SC-point cosine and sine table into shared memory, by the whole CTA
+// (a barrier must follow before its use).
+__device__ __forceinline__ void load_sc(const Tables &T, float4 *sc) {
+    for (int i = threadIdx.x; i < FX_SC; i += blockDim.x) sc[i] = __ldg(T.fxsc + i);
+}
+
+// FP64 form: Z_d = sum_j w_dj exp(i Psi_dj) over bins j0, j0 + stride, .. <= jlast
+// in the split arithmetic of gwns_fx.cuh, each detector's phase by its own
+// frequency term; zh/zl[d][re, im] (double-float, of the scaled data) not reduced
+// over threads. Bound by FP32 and integer issue, about 500 cycles per warp, bin
+// row and three detectors; in FP64 instructions (8 FMAs for the phase, 24 for the
+// sine and cosine, 8 per detector, 64 cycles each) the same took 3600. GB300,
+// 2048 prior draws, batched likelihood: 519,169 bins 84.4 -> 15.3 ms, 64,897 bins
+// 690 -> 169 us; slice update of 4017 bins 9.7 -> 4.3 ms.
+template <int NDET>
+__device__ __forceinline__ void bins_fx(const Tables &T, const FxPoint &c, const float4 *sc, int j0, int stride,
+                                        int jlast, float (&zh)[NDET][2], float (&zl)[NDET][2]) {
+    const int N = T.fxn;
+#pragma unroll
+    for (int d = 0; d < NDET; d++) {
+        zh[d][0] = zh[d][1] = (c.bad && jlast >= 0) ? __int_as_float(0x7fffffff) : 0.f;
+        zl[d][0] = zl[d][1] = 0.f;
+    }
+    if (c.bad) return;
+    fx2 a[NB], t[NDET];
 #pragma unroll
     for (int m = 0; m < NB; m++) a[m] = c.a[m];
-    const double c0 = c.c0;
-    // the thread's bins j_n = tid + n stride, n = 0 .. nb-1; the detector factor
-    // exp(2 pi i f_j tau_d) = R_d rho_d^n with R_d at j_0 and rho_d the rotation
-    // over one stride, so Z_d = R_d sum_n (w_dj exp(i Psi_j)) rho_d^n, evaluated
-    // by Horner's rule from the last bin down: per bin and detector a complex
-    // product and a Horner step (8 FP64) instead of advancing, applying and
-    // accumulating a running phasor (12)
-    const int nb = tid <= c.jcut ? (c.jcut - tid) / stride + 1 : 0;
-    double pr[NDET], pi_[NDET], hr[NDET], hi[NDET];
 #pragma unroll
-    for (int d = 0; d < NDET; d++) {
-        hr[d] = 0.0; hi[d] = 0.0;
-        if (PRE_ROT) {
-            pr[d] = c.rot_re[d];
-            pi_[d] = c.rot_im[d];
-            for (int q = 0; q < rot_sq; q++) {
-                const double re = pr[d] * pr[d] - pi_[d] * pi_[d];
-                pi_[d] = 2.0 * pr[d] * pi_[d];
-                pr[d] = re;
-            }
-        } else if (nb > 0) {
-            sincos_bf(TWO_PI_D * (stride * df) * c.tau[d], pi_[d], pr[d]);
+    for (int d = 0; d < NDET; d++) t[d] = c.t[d];
+    const int64_t c0 = c.c0;
+    const int32_t sh = c.sh;
+#pragma unroll 1
+    for (int j = j0; j <= jlast; j += stride) {
+        int64_t hi = c0, cr = 0;
+#pragma unroll
+        for (int m = 0; m < NB; m += 2) {
+            const int4 b = __ldg(T.fxb + (size_t)(m >> 1) * N + j);
+            fx_mac(hi, cr, a[m], fx2{b.x, b.y});
+            fx_mac(hi, cr, a[m + 1], fx2{b.z, b.w});
         }
-    }
-    for (int n = nb - 1; n >= 0; n--) {
-        const int j = tid + n * stride;
-        double psi = c0;
-#pragma unroll
-        for (int m = 0; m < NB; m++) psi = fma(a[m], __ldg(T.basis64 + (size_t)m * N + j), psi);
-        double s, co;
-        sincos_bf(psi, s, co);
+        const int2 f = __ldg(T.fxf + j);
 #pragma unroll
         for (int d = 0; d < NDET; d++) {
-            const double2 w = __ldg(T.w64 + (size_t)d * N + j);
-            const double cr = fma(w.x, co, -w.y * s), ci = fma(w.x, s, w.y * co);
-            const double h2r = fma(hr[d], pr[d], fma(-hi[d], pi_[d], cr));
-            const double h2i = fma(hr[d], pi_[d], fma(hi[d], pr[d], ci));
-            hr[d] = h2r;
-            hi[d] = h2i;
-        }
-    }
-#pragma unroll
-    for (int d = 0; d < NDET; d++) {
-        zr[d] = 0.0; zi[d] = 0.0;
-        if (nb > 0) {
-            double rs, rc;
-            sincos_bf(TWO_PI_D * (f0 + tid * df) * c.tau[d], rs, rc);
-            zr[d] = rc * hr[d] - rs * hi[d];
-            zi[d] = rc * hi[d] + rs * hr[d];
+            int64_t hd = hi, cd = cr;
+            fx_mac(hd, cd, t[d], fx2{f.x, f.y});
+            const fxe E = fx_cis(fx_phase(hd, cd, sh), sc);
+            fx_cmac(zh[d], zl[d], __ldg(T.fxw + (size_t)d * N + j), E);
         }
     }
 }

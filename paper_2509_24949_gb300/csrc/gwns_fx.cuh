@@ -1,0 +1,184 @@
+// gwns_fx.cuh -- the FP64 form's bin arithmetic off the FP64 pipe. GB300 issues
+// one FP64 warp instruction per 64 cycles per SM sub-partition (measured; FP32
+// one per cycle, a 32 x 32 -> 64-bit integer multiply-add one per four), so a
+// bin's 8 phase terms, its sines and cosines and its complex products cost
+// thousands of cycles in FP64 and a few hundred in the split arithmetic here:
+//
+//  * the phase in turns as a fixed-point sum of products, modulo one turn. The
+//    basis and the frequency are 59-bit integers scaled to their largest value
+//    on the grid, a point's coefficients 58-bit integers on one scale per point
+//    (block floating point: unit 2^-58 of the point's largest term, 32 times
+//    finer than FP64's rounding of that term). Both are split into 30-bit
+//    halves, so that the high and the cross products add up in two 64-bit
+//    accumulators without carries: three multiply-adds per term.
+//  * exp(2 pi i phase): the top 10 fraction bits pick cos and sin of k 2 pi/1024
+//    from a table (double-float, half a turn, the other half by sign), the rest
+//    r, |r| < 0.0031 rad, enters through sin r and cos r - 1 by their Taylor
+//    polynomials and one complex product, all in double-float (absolute error
+//    about 1e-15).
+//  * the products with the weighted data and their sums in double-float
+//    (48 bits), the data scaled by a power of two per detector.
+//
+// Plain C++ besides the qualifiers, so the same code compiles for the host
+// (where a CPU test checks it against 60-digit references) and for sm_103a.
+#pragma once
+#include "gwns_df.cuh"
+
+namespace gwns {
+
+constexpr int FX_NB = 8;            // phase basis functions
+constexpr int FX_DET = 4;           // detectors at most
+constexpr int FX_ABITS = 58;        // coefficients: |A| < 2^58
+constexpr int FX_BBITS = 59;        // tables: |b| <= 2^59
+constexpr int FX_SC = 512;          // table points over half a turn
+
+// A signed 60-bit integer as 2^30 h + l, 0 <= l < 2^30.
+struct fx2 {
+    int32_t h, l;
+};
+
+// One point's fixed-point phase coefficients (a: basis, t: detector delays) in
+// units of 2^(E - 58) turns per full-scale table entry; c0 in the phase sum's
+// unit 2^(E - 57) turns; sh = E + 7 lifts the sum's fraction to 64 bits.
+struct FxPoint {
+    fx2 a[FX_NB];
+    fx2 t[FX_DET];
+    int64_t c0;
+    int32_t sh;
+    int32_t bad;        // a coefficient is not finite: the sums are NaN
+};
+
+struct fxe {
+    float rh, rl, ih, il;       // double-float complex
+};
+
+DFI fx2 fx_split(int64_t v) { return fx2{(int32_t)(v >> 30), (int32_t)(v & 0x3fffffff)}; }
+
+#if defined(__CUDA_ARCH__)
+DFI uint64_t fx_mulhi(uint64_t a, uint64_t b) { return __umul64hi(a, b); }
+DFI uint64_t fx_bits(double x) { return (uint64_t)__double_as_longlong(x); }
+#else
+DFI uint64_t fx_mulhi(uint64_t a, uint64_t b) { return (uint64_t)(((unsigned __int128)a * b) >> 64); }
+DFI uint64_t fx_bits(double x) { uint64_t b; memcpy(&b, &x, 8); return b; }
+#endif
+
+// |x| (or |x| / 2 pi, TURNS) = m 2^e with m a 64-bit integer of at least 62
+// significant bits, from the double's bits alone; 0 (and anything below 2^-1022)
+// gives m = 0. Not finite: *bad is set. Returns e.
+template <bool TURNS>
+DFI int fx_mantissa(double x, uint64_t *m, int32_t *bad) {
+    const uint64_t b = fx_bits(x);
+    const int ex = (int)(b >> 52) & 0x7ff;
+    if (ex == 0x7ff) *bad = 1;
+    if (ex == 0) { *m = 0; return -100000; }
+    const uint64_t q = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
+    // 1/(2 pi) = 0xA2F9836E4E44152A 2^-66 (rounded)
+    *m = TURNS ? fx_mulhi(q, 0xA2F9836E4E44152Aull) : q;
+    return TURNS ? ex - 1088 : ex - 1086;
+}
+// m 2^-s rounded, with x's sign (s >= 1)
+DFI int64_t fx_scaled(uint64_t m, int s, double x) {
+    const uint64_t v = s > 64 ? 0 : ((m >> (s - 1)) + 1) >> 1;
+    return (fx_bits(x) >> 63) ? -(int64_t)v : (int64_t)v;
+}
+
+// Table entry of a double with |v| <= 2^eb.
+#if defined(__CUDACC__)
+__device__ __forceinline__ fx2 fx_table(double v, int eb) {
+    return fx_split(__double2ll_rn(scalbn(v, FX_BBITS - eb)));
+}
+#else
+DFI fx2 fx_table(double v, int eb) { return fx_split(llrint(scalbn(v, FX_BBITS - eb))); }
+#endif
+
+// One term's products: hi += a.h b.h, cr += a.h b.l + a.l b.h (the low product,
+// below the unit, is dropped). |a.h| <= 2^28, |b.h| <= 2^29: the nine terms of a
+// phase stay below 2^62 in either sum.
+DFI void fx_mac(int64_t &hi, int64_t &cr, fx2 a, fx2 b) {
+    hi += (int64_t)a.h * b.h;
+    cr += (int64_t)a.h * b.l;
+    cr += (int64_t)a.l * b.h;
+}
+// The phase's fraction of a turn (2^-64 turns) from the sums.
+DFI uint64_t fx_phase(int64_t hi, int64_t cr, int32_t sh) {
+    const uint64_t p = (uint64_t)(hi + (cr >> 30));
+    return sh > 63 ? 0 : p << sh;
+}
+
+// exp(2 pi i F 2^-64). tab: FX_SC points (cos h, cos l, sin h, sin l) of
+// k 2 pi/1024.
+#if defined(__CUDACC__)
+typedef float4 fx_f4;
+#else
+struct fx_f4 { float x, y, z, w; };
+#endif
+DFI fxe fx_cis(uint64_t F, const fx_f4 *tab) {
+    const uint32_t fh = (uint32_t)(F >> 32), fl = (uint32_t)F;
+    const uint32_t g = fh + 0x200000u;                    // round to the nearest table point
+    // rest in units of 2^-32 turns: r0 = g mod 2^22 - 2^21 (exact) + r1 2^-23
+    const float r0 = f_sub(i_as_f((int32_t)(0x4b000000u | (g & 0x3fffffu))), 10485760.0f);
+    const float r1 = f_sub(i_as_f((int32_t)(0x4b000000u | (fl >> 9))), 8388608.0f);
+    const fx_f4 T = tab[(g >> 22) & (FX_SC - 1)];
+    const uint32_t sgn = g & 0x80000000u;                 // second half turn: -T
+    const float ch = i_as_f((int32_t)((uint32_t)f_as_i(T.x) ^ sgn)), cl = i_as_f((int32_t)((uint32_t)f_as_i(T.y) ^ sgn));
+    const float sh = i_as_f((int32_t)((uint32_t)f_as_i(T.z) ^ sgn)), sl = i_as_f((int32_t)((uint32_t)f_as_i(T.w) ^ sgn));
+    // r = p + e [rad]
+    const float CH = (float)1.4629180792671596e-9, CL = (float)(1.4629180792671596e-9 - (double)CH);   // 2 pi 2^-32
+    const float p = f_mul(r0, CH);
+    float e = f_fma(r0, CH, -p);
+    e = f_fma(r0, CL, e);
+    e = f_fma(r1, (float)(1.4629180792671596e-9 / 8388608.0), e);
+    // cos r - 1 = c1 + c2, sin r = p + s2
+    const float r2 = f_mul(p, p), r2e = f_fma(p, p, -r2);
+    const float c1 = f_mul(-0.5f, r2);
+    const float c2 = f_fma(f_mul(c1, c1), 1.0f / 6.0f, f_fma(-p, e, f_mul(-0.5f, r2e)));
+    const float s2 = f_fma(f_mul(r2, p), f_fma(r2, 1.0f / 120.0f, -1.0f / 6.0f), f_fma(c1, e, e));
+    // T + T (c + i s): the products' sum b (below 0.0031) with the table's low part,
+    // then T + b by size (the table's nonzero entries exceed 0.0061), then the low parts
+    fxe E;
+    {
+        const float u = f_mul(sh, p), ue = f_fma(sh, p, -u);
+        const float v = f_mul(ch, c1), ve = f_fma(ch, c1, -v);
+        const dfl b = two_sum_f(-u, v), bc = two_sum_f(b.h, cl), x = fast_two_sum_f(ch, bc.h);
+        float l = f_add(f_add(b.l, bc.l), f_sub(ve, ue));
+        l = f_fma(ch, c2, l);
+        l = f_fma(-sh, s2, l);
+        l = f_fma(-sl, p, l);
+        l = f_fma(cl, c1, l);
+        E.rh = x.h;
+        E.rl = f_add(x.l, l);
+    }
+    {
+        const float u = f_mul(ch, p), ue = f_fma(ch, p, -u);
+        const float v = f_mul(sh, c1), ve = f_fma(sh, c1, -v);
+        const dfl b = two_sum_f(u, v), bc = two_sum_f(b.h, sl), x = fast_two_sum_f(sh, bc.h);
+        float l = f_add(f_add(b.l, bc.l), f_add(ve, ue));
+        l = f_fma(sh, c2, l);
+        l = f_fma(ch, s2, l);
+        l = f_fma(cl, p, l);
+        l = f_fma(sl, c1, l);
+        E.ih = x.h;
+        E.il = f_add(x.l, l);
+    }
+    return E;
+}
+
+// zh + zl += w E for one real product of double-floats
+DFI void fx_acc(float &zh, float &zl, float wh, float wl, float eh, float el) {
+    const float p = f_mul(wh, eh);
+    float e = f_fma(wh, eh, -p);
+    e = f_fma(wh, el, e);
+    e = f_fma(wl, eh, e);
+    const dfl s = two_sum_f(zh, p);
+    zh = s.h;
+    zl = f_add(zl, f_add(s.l, e));
+}
+// Z += w E, w = (re h, re l, im h, im l), z = (re, im)
+DFI void fx_cmac(float (&zh)[2], float (&zl)[2], fx_f4 w, fxe E) {
+    fx_acc(zh[0], zl[0], w.x, w.y, E.rh, E.rl);
+    fx_acc(zh[0], zl[0], -w.z, -w.w, E.ih, E.il);
+    fx_acc(zh[1], zl[1], w.x, w.y, E.ih, E.il);
+    fx_acc(zh[1], zl[1], w.z, w.w, E.rh, E.rl);
+}
+
+}  // namespace gwns

@@ -167,8 +167,8 @@ __global__ void k_build_tables(Model M, const double *dre, const double *dim, co
             const double sd = psd[o];
             const double wr = 4.0 * M.df * f76 * dre[o] / sd;
             const double wi = 4.0 * M.df * f76 * dim[o] / sd;
-            w64[o] = make_double2(wr, wi);
             const float2 wf = make_float2(__double2float_rn(wr), __double2float_rn(wi));
+            if (w64) w64[o] = make_double2(wr, wi);
             if (lg) {
                 // float2 slot pos of the pair order -> float4 (Re, Re, Im, Im) of its bin pair
                 const size_t pos = (size_t)d * M.np + tile_pos2(j, lg);
@@ -184,23 +184,33 @@ __global__ void k_build_tables(Model M, const double *dre, const double *dim, co
 }
 
 // Inclusive scan of prefix[d][0..N) in place, one block per detector: each
-// thread scans a contiguous chunk, chunk totals are scanned by the block.
+// thread scans a contiguous chunk, chunk totals are scanned by the block (by
+// shuffles: ten roundings deep, where one thread's running sum of the 1024
+// totals took part in <h|h> with a relative error of some 1e-15).
 __global__ void k_prefix_scan(double *prefix, int N) {
     double *p = prefix + (size_t)blockIdx.x * N;
-    __shared__ double tot[1024];
-    const int T = blockDim.x, t = threadIdx.x;
+    __shared__ double tot[32];
+    const int T = blockDim.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int chunk = (N + T - 1) / T;
     const int lo = t * chunk, hi = min(N, lo + chunk);
     double s = 0.0;
     for (int j = lo; j < hi; j++) { s += p[j]; p[j] = s; }
-    tot[t] = s;
-    __syncthreads();
-    if (t == 0) {
-        double acc = 0.0;
-        for (int i = 0; i < T; i++) { double v = tot[i]; tot[i] = acc; acc += v; }
+    double v = s;           // inclusive over the warp
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
     }
+    if (lane == 31) tot[warp] = v;
     __syncthreads();
-    const double off = tot[t];
+    double w = tot[lane];   // every warp scans the (32) warp totals
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += u;
+    }
+    double before = __shfl_up_sync(0xffffffffu, v, 1);
+    if (lane == 0) before = 0.0;
+    const double wb = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+    const double off = (warp > 0 ? wb : 0.0) + before;
     for (int j = lo; j < hi; j++) p[j] += off;
 }
 
@@ -212,6 +222,71 @@ cudaError_t launch_build_tables(const Model &M, const double *data_re, const dou
     k_build_tables<<<blocks, 256, 0, s>>>(M, data_re, data_im, psd, basis64, f64, w64, prefix, X.basis32,
                                           X.f32, X.w32, X.tb0, X.tb1, X.tbk, X.fc, X.wt);
     k_prefix_scan<<<M.n_det, 1024, 0, s>>>(prefix, M.N);
+    return cudaGetLastError();
+}
+
+// FP64 form: the largest |w| of each detector (by the high words of its parts,
+// which order as the magnitudes do; a NaN or infinity wins) ..
+__global__ void k_fx_wmax(const double2 *w64, int N, int n_det, unsigned *wmax) {
+    const int d = blockIdx.y;
+    unsigned mx = 0;
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
+        const double2 w = w64[(size_t)d * N + j];
+        mx = max(mx, max((unsigned)__double2hiint(w.x) & 0x7fffffffu, (unsigned)__double2hiint(w.y) & 0x7fffffffu));
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(wmax + d, mx);
+}
+
+// x as a double-float; infinities and NaN keep their value in h.
+__device__ __forceinline__ float2 fx_df(double x) {
+    const float h = __double2float_rn(x);
+    return make_float2(h, isfinite(h) ? __double2float_rn(x - (double)h) : 0.f);
+}
+
+// .. and the tables: fixed-point basis and frequency, the data scaled by the
+// power of two that takes the detector's largest |w| into [1, 2).
+__global__ void k_build_fx(Model M, Tables T, const double2 *w64, FxTables X) {
+    const int i0 = blockIdx.x * blockDim.x + threadIdx.x, st = gridDim.x * blockDim.x;
+    for (int i = i0; i < FX_SC; i += st) {
+        double sn, cs;
+        sincospi((double)i * (1.0 / FX_SC), &sn, &cs);
+        const float2 c = fx_df(cs), s = fx_df(sn);
+        X.sc[i] = make_float4(c.x, c.y, s.x, s.y);
+    }
+    int e[MAXDET];
+#pragma unroll
+    for (int d = 0; d < MAXDET; d++) {
+        const int ex = d < M.n_det ? (int)(X.wmax[d] >> 20) : 0;
+        e[d] = (ex == 0 || ex == 0x7ff) ? 0 : ex - 1023;
+        if (i0 == 0 && d < M.n_det) X.scale[d] = scalbn(1.0, e[d]);
+    }
+    const int N = M.N;
+    for (int j = i0; j < N; j += st) {
+#pragma unroll
+        for (int m = 0; m < NB; m += 2) {
+            const fx2 a = fx_table(T.basis64[(size_t)m * N + j], T.fxe[m]);
+            const fx2 b = fx_table(T.basis64[(size_t)(m + 1) * N + j], T.fxe[m + 1]);
+            X.b[(size_t)(m >> 1) * X.n + j] = make_int4(a.h, a.l, b.h, b.l);
+        }
+        const fx2 f = fx_table(T.f64[j], T.fxe[NB]);
+        X.f[j] = make_int2(f.h, f.l);
+#pragma unroll
+        for (int d = 0; d < MAXDET; d++) {
+            if (d >= M.n_det) break;
+            const double2 w = w64[(size_t)d * N + j];
+            const float2 re = fx_df(scalbn(w.x, -e[d])), im = fx_df(scalbn(w.y, -e[d]));
+            X.w[(size_t)d * X.n + j] = make_float4(re.x, re.y, im.x, im.y);
+        }
+    }
+}
+
+cudaError_t launch_build_fx(const Model &M, const Tables &T, const double2 *w64, const FxTables &X, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(X.wmax, 0, sizeof(unsigned) * M.n_det, s);
+    if (e != cudaSuccess) return e;
+    const int blocks = min((M.N + 255) / 256, 152 * 4);
+    k_fx_wmax<<<dim3(blocks, M.n_det), 256, 0, s>>>(w64, M.N, M.n_det, X.wmax);
+    k_build_fx<<<min((max(M.N, FX_SC) + 127) / 128, 152 * 8), 128, 0, s>>>(M, T, w64, X);
     return cudaGetLastError();
 }
 

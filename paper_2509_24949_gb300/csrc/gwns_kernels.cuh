@@ -95,6 +95,17 @@ __device__ __forceinline__ void load_desc(const Desc *g, Desc &s) {
     __syncthreads();
 }
 
+// Writable tables of the FP64 form's split arithmetic (Tables::fxb .. fxsc).
+struct FxTables {
+    int4 *b;
+    int2 *f;
+    float4 *w;
+    double *scale;
+    float4 *sc;
+    unsigned *wmax;     // [n_det] largest |w|'s high word (scratch of the build)
+    int n;              // rows
+};
+
 // Writable mixed-form tables (per-bin or tiled set, by Model::tlg).
 struct MixedTables {
     float2 *basis32, *f32, *w32;
@@ -141,6 +152,8 @@ int ws_blocks_per_sm(int precision, int ndet);
 cudaError_t launch_build_tables(const Model &M, const double *data_re, const double *data_im,
                                 const double *psd, double *basis64, double *f64, double2 *w64,
                                 double *prefix, const MixedTables &X, cudaStream_t s);
+// The FP64 form's split tables from the grid's basis64, f64 and w64 (exponents: Tables::fxe).
+cudaError_t launch_build_fx(const Model &M, const Tables &T, const double2 *w64, const FxTables &X, cudaStream_t s);
 cudaError_t launch_init_live(const Model &M, uint64_t seed, int n, double *live_u, cudaStream_t s);
 cudaError_t launch_eval(const Model &M, const Tables &T, int precision, int warps, const double *in,
                         int in_is_theta, int m, double *logl, RunState *st, cudaStream_t s);

@@ -9,10 +9,11 @@ namespace gwns {
 
 // The warp sums of one candidate's double-float sums zh/zl[d][re, im] by the
 // transposing butterfly (warp_sum_df_many; lanes 2v hold value v = 2 d + re/im),
-// written as doubles to out[v] (2 NDET entries).
+// written as doubles to out[v] (2 NDET entries), times the detector's data scale
+// where there is one.
 template <int NDET>
 __device__ __forceinline__ void warp_sums_df_to(const float (&zh)[NDET][2], const float (&zl)[NDET][2],
-                                                double *out) {
+                                                double *out, const double *scale = nullptr) {
     const int lane = threadIdx.x & 31;
     float vh[16], vl[16];
 #pragma unroll
@@ -22,7 +23,10 @@ __device__ __forceinline__ void warp_sums_df_to(const float (&zh)[NDET][2], cons
     float rh, rl;
     warp_sum_df_many<2 * NDET>(vh, vl, rh, rl);
     const int v = lane >> 1;
-    if ((lane & 1) == 0 && v < 2 * NDET) out[v] = (double)rh + (double)rl;
+    if ((lane & 1) == 0 && v < 2 * NDET) {
+        const double z = (double)rh + (double)rl;
+        out[v] = scale ? z * __ldg(scale + (v >> 1)) : z;
+    }
 }
 
 // The same sums combined with G_d: returns sum_d (Re G_d Re Z_d - gim_d Im Z_d)
@@ -30,7 +34,7 @@ __device__ __forceinline__ void warp_sums_df_to(const float (&zh)[NDET][2], cons
 // lane holding value v multiplies it by its factor, then lanes 0, 2, .., 14 add.
 template <int NDET>
 __device__ __forceinline__ double warp_detector_terms_df(const float (&zh)[NDET][2], const float (&zl)[NDET][2],
-                                                         const Coef &c) {
+                                                         const Coef &c, const double *scale = nullptr) {
     const int lane = threadIdx.x & 31;
     float vh[16], vl[16];
 #pragma unroll
@@ -42,7 +46,8 @@ __device__ __forceinline__ double warp_detector_terms_df(const float (&zh)[NDET]
     const int v = lane >> 1, dd = v >> 1;
     double t = 0.0;
     if ((lane & 1) == 0 && v < 2 * NDET) {
-        const double z = (double)rh + (double)rl;
+        double z = (double)rh + (double)rl;
+        if (scale) z *= __ldg(scale + dd);
         t = (v & 1) ? -c.gim[dd] * z : c.gre[dd] * z;
     }
 #pragma unroll
@@ -54,17 +59,18 @@ __device__ __forceinline__ double warp_detector_terms_df(const float (&zh)[NDET]
 // loop and the CTA reduces Z_d. Returns log L in *lval (shared) after the
 // second barrier; every thread of the CTA must call it.
 template <int PREC, int NDET, int W>
-__device__ __forceinline__ void cta_loglike_bins(const Model &M, const Tables &T, Coef &coef,
-                                                 CoefMixed &cm, double (*red)[2 * MAXDET], double *lval) {
+__device__ __forceinline__ void cta_loglike_bins(const Model &M, const Tables &T, Coef &coef, CoefMixed &cm,
+                                                 const FxPoint &fx, const float4 *sc, double (*red)[2 * MAXDET],
+                                                 double *lval) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double zr[NDET], zi[NDET];
+    if (M.model == M_TOY) {
+        if (threadIdx.x == 0) *lval = coef.toy;
+        return;
+    }
     if (PREC == 0) {
-        bins_fp64<NDET>(T, M.N, M.f0, M.df, coef, threadIdx.x, W * 32, zr, zi);
-#pragma unroll
-        for (int d = 0; d < NDET; d++) {
-            zr[d] = warp_sum(zr[d]);
-            zi[d] = warp_sum(zi[d]);
-        }
+        float zh[NDET][2], zl[NDET][2];
+        bins_fx<NDET>(T, fx, sc, threadIdx.x, W * 32, coef.jcut, zh, zl);
+        warp_sums_df_to<NDET>(zh, zl, red[warp], T.fxs);
     } else if (M.tlg) {
         // tiled form: warp w takes tile groups w, w + W, ...
         float zh[1][NDET][2], zl[1][NDET][2];
@@ -78,10 +84,6 @@ __device__ __forceinline__ void cta_loglike_bins(const Model &M, const Tables &T
         bins_mixed<NDET>(T, M.N, cm, coef.jcut, threadIdx.x, W * 32, zh, zl);
         warp_sums_df_to<NDET>(zh, zl, red[warp]);
     }
-    if (PREC == 0 && lane == 0) {
-#pragma unroll
-        for (int d = 0; d < NDET; d++) { red[warp][2 * d] = zr[d]; red[warp][2 * d + 1] = zi[d]; }
-    }
     __syncthreads();
     if (warp == 0) {
         double v = 0.0;
@@ -91,7 +93,7 @@ __device__ __forceinline__ void cta_loglike_bins(const Model &M, const Tables &T
             v = coef.gre[lane] * ZR - coef.gim[lane] * ZI;
         }
         v = warp_sum(v);
-        if (lane == 0) *lval = (M.model == M_TOY) ? coef.toy : v - 0.5 * coef.hh;
+        if (lane == 0) *lval = v - 0.5 * coef.hh;
     }
 }
 
@@ -99,8 +101,7 @@ __device__ __forceinline__ void cta_loglike_bins(const Model &M, const Tables &T
 // (or physical parameters theta when in_is_theta).
 __device__ __forceinline__ void warp_point_coef(const Model &M, const Tables &T, const double *in,
                                                 int in_is_theta, int precision, Coef *coef,
-                                                CoefMixed *cm) {
-    const int lane = threadIdx.x & 31;
+                                                CoefMixed *cm, FxPoint *fx) {
     if (M.model == M_TOY) {
         point_coef_warp(M, T, in, coef);
         return;
@@ -120,7 +121,7 @@ __device__ __forceinline__ void warp_point_coef(const Model &M, const Tables &T,
     }
     __syncwarp();
     if (precision == 1) coef_to_mixed_warp(*coef, M.n_det, M.df, cm, M.rb ? T.rb.fid : nullptr, M.tlg >= 5);
-    (void)lane;
+    else if (!M.rb) coef_to_fx_group(T, M.n_det, coef, fx, 1);
 }
 
 // Points per CTA of the batched likelihood: the coefficient stage packs up to
@@ -139,8 +140,11 @@ __global__ void __launch_bounds__(W * 32) k_eval(Model M, Tables T, const double
     __shared__ double red[W][2 * MAXDET];
     __shared__ double lval;
     __shared__ double pt[EVAL_PPC][NPARAM + MAXD];
+    __shared__ FxPoint fx;
+    __shared__ float4 sc[PREC == 0 ? FX_SC : 1];
     const int i0 = blockIdx.x * ppc;
     if (i0 >= m) return;
+    if (PREC == 0 && M.model == M_GW && !M.rb) load_sc(T, sc);
     const int np = m - i0 < ppc ? m - i0 : ppc;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stride_in = in_is_theta ? NPARAM : M.dim;
@@ -149,9 +153,9 @@ __global__ void __launch_bounds__(W * 32) k_eval(Model M, Tables T, const double
     __syncthreads();
     if (warp == 0) {
         if (ppc == 1) {
-            warp_point_coef(M, T, pt[0], in_is_theta, PREC, &coef[0], &cm[0]);
+            warp_point_coef(M, T, pt[0], in_is_theta, PREC, &coef[0], &cm[0], &fx);
         } else {
-            point_coef_group(M, T, pt[0], NPARAM + MAXD, coef, np, 0);
+            point_coef_group(M, T, pt[0], NPARAM + MAXD, coef, np);
             __syncwarp();
             if (PREC == 1)
                 for (int p = 0; p < np; p++)
@@ -171,7 +175,7 @@ __global__ void __launch_bounds__(W * 32) k_eval(Model M, Tables T, const double
             }
             continue;
         }
-        cta_loglike_bins<PREC, NDET, W>(M, T, coef[p], cm[p], red, &lval);
+        cta_loglike_bins<PREC, NDET, W>(M, T, coef[p], cm[p], fx, sc, red, &lval);
         if (threadIdx.x == 0) {
             logl[i0 + p] = lval;
             if (st) {
@@ -223,7 +227,7 @@ __global__ void __launch_bounds__(W * 32) k_eval_batch(Model M, Tables T, const 
             point_coef_group_mx(M, T, pt[4 * grp], MAXD, &coef[4 * grp], &cm[4 * grp], cnt, M.tlg >= 5,
                                 W >= 2 ? 1 + (warp & 1) : 0);
         else
-            point_coef_group(M, T, pt[4 * grp], MAXD, &coef[4 * grp], cnt, 0, W >= 2 ? 1 + (warp & 1) : 0);
+            point_coef_group(M, T, pt[4 * grp], MAXD, &coef[4 * grp], cnt, W >= 2 ? 1 + (warp & 1) : 0);
     }
     __syncthreads();
     if (cnt > 0 && lead) {
@@ -847,8 +851,12 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
     __shared__ int e_next_step, cur_step;
     __shared__ int jc[S];
     __shared__ double part[W][S][NDET][2];
+    __shared__ FxPoint fx[PREC == 0 ? S : 1];
+    __shared__ float4 sct[PREC == 0 ? FX_SC : 1];
     if (chain >= A.k) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d = M.dim;
+    const bool use_fx = PREC == 0 && M.model == M_GW && !M.rb;
+    if (use_fx) load_sc(T, sct);    // used after the first round's barriers
     const uint32_t iter = (uint32_t)A.state->iter;
     const double lstar = A.state->lstar;
     const int walk_len = A.state->walk_len;
@@ -918,8 +926,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                     point_coef_group_mx(M, T, ysh[4 * grp], MAXD, &coef[4 * grp], &cm[4 * grp], cnt,
                                         form_rot<FORM>(M), 1 + (warp & 1));
                 else
-                    point_coef_group(M, T, ysh[4 * grp], MAXD, &coef[4 * grp], cnt, PREC == 0 ? 32 : 0,
-                                     1 + (warp & 1));
+                    point_coef_group(M, T, ysh[4 * grp], MAXD, &coef[4 * grp], cnt, 1 + (warp & 1));
             } else if (warp == W - 1 && A.kernel == 0) {
                 // a warp without coefficients computes the next slice step's direction
                 const int s1 = cur_step + 1;
@@ -934,6 +941,9 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             }
             __syncthreads();
             if (warp == 0) point_coef_join(M, T, coef, ns);
+            // meanwhile the odd warp of each group of four: the fixed-point coefficients
+            if (use_fx && (warp & 1) && 4 * grp < ns)
+                coef_to_fx_group(T, M.n_det, &coef[4 * grp], &fx[4 * grp], min(4, ns - 4 * grp));
             __syncthreads();
         } else {
             if (4 * warp < ns) {
@@ -942,7 +952,11 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                     point_coef_group_mx(M, T, ysh[4 * warp], MAXD, &coef[4 * warp], &cm[4 * warp], cnt,
                                         form_rot<FORM>(M));
                 else
-                    point_coef_group(M, T, ysh[4 * warp], MAXD, &coef[4 * warp], cnt, PREC == 0 ? 32 : 0);
+                    point_coef_group(M, T, ysh[4 * warp], MAXD, &coef[4 * warp], cnt);
+                if (use_fx) {
+                    __syncwarp();
+                    coef_to_fx_group(T, M.n_det, &coef[4 * warp], &fx[4 * warp], cnt);
+                }
             }
             __syncthreads();
         }
@@ -1035,13 +1049,9 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             const int lg = 1;
             const int wpc = 1 << lg, cand = warp >> lg, sub = warp & (wpc - 1);
             if (cand < ns) {
-                double zr[NDET], zi[NDET];
-                bins_fp64<NDET, true>(T, M.N, M.f0, M.df, coef[cand], sub * 32 + lane, wpc * 32, zr, zi, lg);
-#pragma unroll
-                for (int dd = 0; dd < NDET; dd++) {
-                    const double ZR = warp_sum(zr[dd]), ZI = warp_sum(zi[dd]);
-                    if (lane == 0) { part[warp][0][dd][0] = ZR; part[warp][0][dd][1] = ZI; }
-                }
+                float zh[NDET][2], zl[NDET][2];
+                bins_fx<NDET>(T, fx[cand], sct, sub * 32 + lane, wpc * 32, coef[cand].jcut, zh, zl);
+                warp_sums_df_to<NDET>(zh, zl, &part[warp][0][0][0], T.fxs);
             }
             __syncthreads();
             if (warp == 0) {
@@ -1063,12 +1073,10 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             // one candidate per slot warp: bins and warp reduction
             double v = 0.0;
             if (PREC == 0) {
-                double zr[NDET], zi[NDET];
-                bins_fp64<NDET, true>(T, M.N, M.f0, M.df, coef[warp], lane, 32, zr, zi);
-#pragma unroll
-                for (int dd = 0; dd < NDET; dd++) {
-                    const double ZR = warp_sum(zr[dd]), ZI = warp_sum(zi[dd]);
-                    v += coef[warp].gre[dd] * ZR - coef[warp].gim[dd] * ZI;
+                if (use_fx) {
+                    float zh[NDET][2], zl[NDET][2];
+                    bins_fx<NDET>(T, fx[warp], sct, lane, 32, coef[warp].jcut, zh, zl);
+                    v = warp_detector_terms_df<NDET>(zh, zl, coef[warp], T.fxs);
                 }
             } else if (M.tlg) {
                 if (!M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, form_rot<FORM>(M));
