@@ -96,6 +96,9 @@ struct Tables {
     const double *fxs;       // [n_det]   power-of-two scale of the weighted data
     const float4 *fxsc;      // [FX_SC]   cos and sin of k 2 pi/1024, double-float
     int fxn;                 // rows of fxb, fxf and fxw
+    FxTiles tiles;           // node rows after the bins' (long grids)
+    // the points that the tiles serve: |a_m - box_a[m]| <= box_r[m], |tau_d - box_a[NB]| <= box_r[NB]
+    double box_a[NB + 1], box_r[NB + 1];
     int fxe[NB + 1];         // binary exponents of the basis functions' and the frequency's scale
     const double *prefix;    // [n_det][N] P_d(j)
     // mixed form, per bin (Model::tlg == 0)
@@ -802,6 +805,11 @@ __device__ inline void coef_to_fx_group(const Tables &T, int n_det, const Coef *
     const int ea = fx_mantissa<true>(a, &ma, &bad) + T.fxe[sl];
     const int et = fx_mantissa<false>(tau, &mt, &bad) + T.fxe[NB];
     const int ec = fx_mantissa<true>(ph, &mc, &bad);
+    // inside the tiles' box? (a NaN is not)
+    bool in = true;
+    if (T.tiles.nlev > 0)
+        in = fabs(a - T.box_a[sl]) <= T.box_r[sl] && (!det || fabs(tau - T.box_a[NB]) <= T.box_r[NB]);
+    in = ((__ballot_sync(0xffffffffu, in) >> (lane & 24)) & 0xffu) == 0xffu;
     // the point's scale 2^E: above every term's largest value on the grid
     int E = max(max(max(ea, et), ec) + 64, 0);
 #pragma unroll
@@ -816,6 +824,7 @@ __device__ inline void coef_to_fx_group(const Tables &T, int n_det, const Coef *
         o.c0 = fx_scaled(mc, E - (ec + 64) + 7, ph);
         o.sh = E + 7;
         o.bad = bad;
+        fx_segments(T.tiles, in, c.jcut + 1, o);
     }
 }
 
@@ -825,7 +834,7 @@ __device__ __forceinline__ void load_sc(const Tables &T, float4 *sc) {
     for (int i = threadIdx.x; i < FX_SC; i += blockDim.x) sc[i] = __ldg(T.fxsc + i);
 }
 
-// FP64 form: Z_d = sum_j w_dj exp(i Psi_dj) over bins j0, j0 + stride, .. <= jlast
+// FP64 form: Z_d = sum_j w_dj exp(i Psi_dj) over the point's rows j0, j0 + stride, ..
 // in the split arithmetic of gwns_fx.cuh, each detector's phase by its own
 // frequency term; zh/zl[d][re, im] (double-float, of the scaled data) not reduced
 // over threads. Bound by FP32 and integer issue, about 500 cycles per warp, bin
@@ -835,11 +844,11 @@ __device__ __forceinline__ void load_sc(const Tables &T, float4 *sc) {
 // 690 -> 169 us; slice update of 4017 bins 9.7 -> 4.3 ms.
 template <int NDET>
 __device__ __forceinline__ void bins_fx(const Tables &T, const FxPoint &c, const float4 *sc, int j0, int stride,
-                                        int jlast, float (&zh)[NDET][2], float (&zl)[NDET][2]) {
-    const int N = T.fxn;
+                                        float (&zh)[NDET][2], float (&zl)[NDET][2]) {
+    const int N = T.fxn, rows = c.rows;
 #pragma unroll
     for (int d = 0; d < NDET; d++) {
-        zh[d][0] = zh[d][1] = (c.bad && jlast >= 0) ? __int_as_float(0x7fffffff) : 0.f;
+        zh[d][0] = zh[d][1] = (c.bad && rows > 0) ? __int_as_float(0x7fffffff) : 0.f;
         zl[d][0] = zl[d][1] = 0.f;
     }
     if (c.bad) return;
@@ -850,8 +859,11 @@ __device__ __forceinline__ void bins_fx(const Tables &T, const FxPoint &c, const
     for (int d = 0; d < NDET; d++) t[d] = c.t[d];
     const int64_t c0 = c.c0;
     const int32_t sh = c.sh;
+    int seg = 0;
 #pragma unroll 1
-    for (int j = j0; j <= jlast; j += stride) {
+    for (int r = j0; r < rows; r += stride) {
+        while (r >= c.seg[seg].end) seg++;
+        const int j = r + c.seg[seg].off;
         int64_t hi = c0, cr = 0;
 #pragma unroll
         for (int m = 0; m < NB; m += 2) {

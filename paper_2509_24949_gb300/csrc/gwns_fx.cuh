@@ -31,6 +31,10 @@ constexpr int FX_DET = 4;           // detectors at most
 constexpr int FX_ABITS = 58;        // coefficients: |A| < 2^58
 constexpr int FX_BBITS = 59;        // tables: |b| <= 2^59
 constexpr int FX_SC = 512;          // table points over half a turn
+constexpr int FX_NODES = 32;        // nodes of a tile (below)
+constexpr int FX_LG0 = 6;           // log2 of the shortest tile's bins
+constexpr int FX_LEV = 10;          // tile levels at most
+constexpr int FX_SEG = 2 * FX_LEV + 1;
 
 // A signed 60-bit integer as 2^30 h + l, 0 <= l < 2^30.
 struct fx2 {
@@ -46,6 +50,22 @@ struct FxPoint {
     int64_t c0;
     int32_t sh;
     int32_t bad;        // a coefficient is not finite: the sums are NaN
+    // the rows to sum: running index r < rows lies in the first segment with
+    // r < end and is table row r + off
+    int32_t nseg, rows;
+    struct { int32_t end, off; } seg[FX_SEG];
+};
+
+// Tiles of the long grids. Over a tile of 2^(FX_LG0 + l) bins (level l) the
+// phase of any point of the prior differs from a reference phase by a few
+// radians, so exp(i (Psi - Psi_ref)) is a polynomial of degree 31 there to 1e-15
+// and the tile's sum over bins is exactly a sum over FX_NODES Chebyshev nodes,
+// with the bins' weighted data gathered once into weights of the nodes. Level l
+// covers the grid from bin first[l] on (where its bound holds) with rows from
+// row[l] on; rows 0 .. N-1 are the bins themselves.
+struct FxTiles {
+    int32_t nlev;
+    int32_t first[FX_LEV], row[FX_LEV];
 };
 
 struct fxe {
@@ -90,6 +110,45 @@ __device__ __forceinline__ fx2 fx_table(double v, int eb) {
 #else
 DFI fx2 fx_table(double v, int eb) { return fx_split(llrint(scalbn(v, FX_BBITS - eb))); }
 #endif
+
+// The segments of the bins 0 .. n - 1: bins below the first tiled one, then tiles
+// of growing length, each level up to the next one's first bin, then of
+// shrinking length up to the cutoff and the last few bins one by one.
+DFI void fx_segments(const FxTiles &T, bool tiles, int n, FxPoint &o) {
+    int ns = 0, rows = 0, pos = 0;
+    if (tiles && T.nlev > 0 && n > T.first[0]) {
+        if (T.first[0] > 0) {
+            pos = rows = T.first[0];
+            o.seg[ns].end = rows;
+            o.seg[ns++].off = 0;
+        }
+        int l = 0, step = 1;
+        for (int it = 0; it < 2 * FX_LEV && l >= 0; it++) {
+            const int lg = FX_LG0 + l;
+            int e = n >> lg << lg;
+            bool up = false;
+            if (step > 0 && l + 1 < T.nlev && e >= T.first[l + 1]) {
+                e = T.first[l + 1];
+                up = true;
+            }
+            if (e > pos) {
+                o.seg[ns].off = T.row[l] + ((pos - T.first[l]) >> lg) * FX_NODES - rows;
+                rows += ((e - pos) >> lg) * FX_NODES;
+                o.seg[ns++].end = rows;
+                pos = e;
+            }
+            if (!up) step = -1;
+            l += step;
+        }
+    }
+    if (n > pos) {
+        o.seg[ns].off = pos - rows;
+        rows += n - pos;
+        o.seg[ns++].end = rows;
+    }
+    o.nseg = ns;
+    o.rows = rows;
+}
 
 // One term's products: hi += a.h b.h, cr += a.h b.l + a.l b.h (the low product,
 // below the unit, is dropped). |a.h| <= 2^28, |b.h| <= 2^29: the nine terms of a

@@ -281,12 +281,114 @@ __global__ void k_build_fx(Model M, Tables T, const double2 *w64, FxTables X) {
     }
 }
 
+// Prior draws' phase coefficients and cutoffs, for the tiles' box: draw i < 16 has the
+// chirp mass, mass ratio and spins at the ends of their ranges by the bits of i.
+__global__ void __launch_bounds__(256) k_prior_coefs(Model M, Tables T, int m, Coef *out) {
+    __shared__ double u[32][MAXD];
+    const int base = blockIdx.x * 32, warp = threadIdx.x >> 5;
+    for (int t = threadIdx.x; t < 32 * MAXD; t += 256) {
+        const int i = base + t / MAXD, c = t % MAXD;
+        const uint4 w = draw(0x5eedull, (uint32_t)c, 0u, (uint32_t)i, 0u);
+        u[t / MAXD][c] = u01(w.x, w.y);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < 32; t += 256)
+        if (base + t < 16)
+            for (int b = 0; b < 4; b++) {
+                const int p = b == 0 ? P_MC : b == 1 ? P_Q : b == 2 ? P_CHI1 : P_CHI2;
+                if (M.kind[p] != K_FIXED) u[t][M.uidx[p]] = (double)(((base + t) >> b) & 1);
+            }
+    __syncthreads();
+    const int n = min(4, m - base - 4 * warp);
+    if (n > 0) point_coef_group(M, T, u[4 * warp], MAXD, out + base + 4 * warp, n, 1);
+}
+
+cudaError_t launch_prior_coefs(const Model &M, const Tables &T, int m, Coef *out, cudaStream_t s) {
+    k_prior_coefs<<<(m + 31) / 32, 256, 0, s>>>(M, T, m, out);
+    return cudaGetLastError();
+}
+
+// The node rows of one tile level, one CTA per tile (32 threads per detector).
+// With the reference phase taken out, a tile's sum over its sources x (a shortest
+// tile's bins; a longer tile's halves' nodes) is sum_n E(f_n) V_n with
+// V_n = sum_x l_n(x) v_x, l_n the nodes' Lagrange polynomials: 64 sources, 32 nodes.
+// The row's weight is V_n with the reference phase put back at the node.
+__global__ void k_fx_nodes(Model M, Tables T, const double2 *w64, FxTables X, int lev, const double2 *vsrc,
+                           double2 *vdst) {
+    __shared__ double2 src[2 * FX_NODES][MAXDET];
+    __shared__ double2 back[FX_NODES];
+    const int nd = M.n_det, lg = FX_LG0 + lev, tile = blockIdx.x;
+    const int s = T.tiles.first[lev] + (tile << lg);
+    const size_t row0 = (size_t)T.tiles.row[lev] + (size_t)tile * FX_NODES;
+    const int n = threadIdx.x & 31, dd = threadIdx.x >> 5;
+    if (lev == 0) {
+        for (int i = threadIdx.x; i < 2 * FX_NODES; i += blockDim.x) {
+            const int j = s + i;
+            int64_t hi = X.ref.c0, cr = 0;
+            for (int m = 0; m < NB; m += 2) {
+                const int4 b = X.b[(size_t)(m >> 1) * X.n + j];
+                fx_mac(hi, cr, X.ref.a[m], fx2{b.x, b.y});
+                fx_mac(hi, cr, X.ref.a[m + 1], fx2{b.z, b.w});
+            }
+            const int2 f = X.f[j];
+            fx_mac(hi, cr, X.ref.t[0], fx2{f.x, f.y});
+            const fxe E = fx_cis(fx_phase(hi, cr, X.ref.sh), X.sc);
+            const double er = (double)E.rh + (double)E.rl, ei = (double)E.ih + (double)E.il;
+            for (int d = 0; d < nd; d++) {
+                const double2 w = w64[(size_t)d * M.N + j];
+                src[i][d] = make_double2(w.x * er - w.y * ei, w.x * ei + w.y * er);
+            }
+        }
+    } else {
+        const size_t o = (size_t)((s - T.tiles.first[lev - 1]) >> (lg - 1)) * FX_NODES * nd;
+        for (int i = threadIdx.x; i < 2 * FX_NODES * nd; i += blockDim.x) src[i / nd][i % nd] = vsrc[o + i];
+    }
+    if (dd == 0) {
+        // the node: interval of half-width L/2 bins about the tile's centre
+        const double L = (double)(1 << lg);
+        const double x = (double)s + 0.5 * (L - 1.0) + 0.5 * L * cospi((2 * n + 1) / (2.0 * FX_NODES));
+        const double f = fma(x, M.df, M.f0);
+        double B[NB];
+        basis_at(f, B);
+        int64_t hi = X.ref.c0, cr = 0;
+#pragma unroll
+        for (int m = 0; m < NB; m += 2) {
+            const fx2 a = fx_table(B[m], T.fxe[m]), b = fx_table(B[m + 1], T.fxe[m + 1]);
+            X.b[(size_t)(m >> 1) * X.n + row0 + n] = make_int4(a.h, a.l, b.h, b.l);
+            fx_mac(hi, cr, X.ref.a[m], a);
+            fx_mac(hi, cr, X.ref.a[m + 1], b);
+        }
+        const fx2 ff = fx_table(f, T.fxe[NB]);
+        X.f[row0 + n] = make_int2(ff.h, ff.l);
+        fx_mac(hi, cr, X.ref.t[0], ff);
+        const fxe E = fx_cis(fx_phase(hi, cr, X.ref.sh), X.sc);
+        back[n] = make_double2((double)E.rh + (double)E.rl, -((double)E.ih + (double)E.il));
+    }
+    __syncthreads();
+    const double *lag = lev == 0 ? X.lag0 : X.lag1;
+    double vr = 0.0, vi = 0.0;
+    for (int i = 0; i < 2 * FX_NODES; i++) {
+        const double l = lag[i * FX_NODES + n];
+        vr = fma(l, src[i][dd].x, vr);
+        vi = fma(l, src[i][dd].y, vi);
+    }
+    vdst[((size_t)tile * FX_NODES + n) * nd + dd] = make_double2(vr, vi);
+    const double2 b = back[n];
+    const double sc = 1.0 / X.scale[dd];        // a power of two
+    const float2 re = fx_df((vr * b.x - vi * b.y) * sc), im = fx_df((vr * b.y + vi * b.x) * sc);
+    X.w[(size_t)dd * X.n + row0 + n] = make_float4(re.x, re.y, im.x, im.y);
+}
+
 cudaError_t launch_build_fx(const Model &M, const Tables &T, const double2 *w64, const FxTables &X, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(X.wmax, 0, sizeof(unsigned) * M.n_det, s);
     if (e != cudaSuccess) return e;
     const int blocks = min((M.N + 255) / 256, 152 * 4);
     k_fx_wmax<<<dim3(blocks, M.n_det), 256, 0, s>>>(w64, M.N, M.n_det, X.wmax);
     k_build_fx<<<min((max(M.N, FX_SC) + 127) / 128, 152 * 8), 128, 0, s>>>(M, T, w64, X);
+    for (int l = 0; l < T.tiles.nlev; l++) {
+        const int tiles = (M.N - T.tiles.first[l]) >> (FX_LG0 + l);
+        k_fx_nodes<<<tiles, 32 * M.n_det, 0, s>>>(M, T, w64, X, l, X.v[(l + 1) & 1], X.v[l & 1]);
+    }
     return cudaGetLastError();
 }
 

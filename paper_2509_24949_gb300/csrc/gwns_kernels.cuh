@@ -104,6 +104,12 @@ struct FxTables {
     float4 *sc;
     unsigned *wmax;     // [n_det] largest |w|'s high word (scratch of the build)
     int n;              // rows
+    // tiles: the reference point, the interpolation matrices [position][node] of a
+    // shortest tile's bins and of a tile's two halves' nodes, and two levels'
+    // node weights in FP64 (scratch of the build)
+    FxPoint ref;
+    double *lag0, *lag1;
+    double2 *v[2];
 };
 
 // Writable mixed-form tables (per-bin or tiled set, by Model::tlg).
@@ -153,6 +159,8 @@ cudaError_t launch_build_tables(const Model &M, const double *data_re, const dou
                                 const double *psd, double *basis64, double *f64, double2 *w64,
                                 double *prefix, const MixedTables &X, cudaStream_t s);
 // The FP64 form's split tables from the grid's basis64, f64 and w64 (exponents: Tables::fxe).
+// Phase coefficients of m prior draws (the first 16 at the corners of the mass and spin ranges).
+cudaError_t launch_prior_coefs(const Model &M, const Tables &T, int m, Coef *out, cudaStream_t s);
 cudaError_t launch_build_fx(const Model &M, const Tables &T, const double2 *w64, const FxTables &X, cudaStream_t s);
 cudaError_t launch_init_live(const Model &M, uint64_t seed, int n, double *live_u, cudaStream_t s);
 cudaError_t launch_eval(const Model &M, const Tables &T, int precision, int warps, const double *in,

@@ -69,7 +69,7 @@ __device__ __forceinline__ void cta_loglike_bins(const Model &M, const Tables &T
     }
     if (PREC == 0) {
         float zh[NDET][2], zl[NDET][2];
-        bins_fx<NDET>(T, fx, sc, threadIdx.x, W * 32, coef.jcut, zh, zl);
+        bins_fx<NDET>(T, fx, sc, threadIdx.x, W * 32, zh, zl);
         warp_sums_df_to<NDET>(zh, zl, red[warp], T.fxs);
     } else if (M.tlg) {
         // tiled form: warp w takes tile groups w, w + W, ...
@@ -266,6 +266,68 @@ __global__ void __launch_bounds__(W * 32) k_eval_batch(Model M, Tables T, const 
     }
 }
 
+// Batched likelihood, FP64, unit-cube points: the CTA's warps take as many points
+// at most. The coefficient stage, bound by the FP64 pipe and its latency (about 250 dependent
+// instructions for up to four points in a warp's lane groups), runs as its two
+// halves on two warps per four points; then the warps share the P C items
+// (point, C-th part of its bin rows), reduced in double-float, and one lane per
+// (point, detector) adds the parts in order. C depends on the grid alone, so a
+// point's log L does not depend on the batch it comes in. GB300, one point per CTA
+// with its coefficients on one warp -> this kernel: 1000 draws of 4017 bins 55.7 ->
+// 47.2 us, 64 draws of 512 bins 36.6 -> 32.5 us (8 warps a CTA: 50.5 and 38.1).
+constexpr int EVAL_FX_W = 4;                // warps
+constexpr int EVAL_FX_P = EVAL_FX_W;        // points at most
+
+template <int NDET>
+__global__ void __launch_bounds__(EVAL_FX_W * 32, 16 / EVAL_FX_W) k_eval_fx(Model M, Tables T, const double *in,
+                                                                            int m, int P, int C, double *logl,
+                                                                            RunState *st) {
+    __shared__ Coef coef[EVAL_FX_P];
+    __shared__ FxPoint fx[EVAL_FX_P];
+    __shared__ float4 sc[FX_SC];
+    __shared__ double pt[EVAL_FX_P][MAXD];
+    __shared__ double red[EVAL_FX_P][8][2 * NDET];
+    const int i0 = blockIdx.x * P;
+    if (i0 >= m) return;
+    const int np = m - i0 < P ? m - i0 : P;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d = M.dim;
+    for (int t = threadIdx.x; t < np * d; t += EVAL_FX_W * 32) pt[t / d][t % d] = in[(size_t)i0 * d + t];
+    load_sc(T, sc);
+    __syncthreads();
+    const int grp = warp >> 1, cnt = 4 * grp < np ? min(4, np - 4 * grp) : 0;
+    if (cnt > 0) point_coef_group(M, T, pt[4 * grp], MAXD, &coef[4 * grp], cnt, 1 + (warp & 1));
+    __syncthreads();
+    if (cnt > 0) {
+        if (warp & 1) coef_to_fx_group(T, M.n_det, &coef[4 * grp], &fx[4 * grp], cnt);
+        else point_coef_join(M, T, &coef[4 * grp], cnt);
+    }
+    __syncthreads();
+    for (int it = warp; it < np * C; it += EVAL_FX_W) {
+        const int p = it / C, c = it - p * C;
+        float zh[NDET][2], zl[NDET][2];
+        bins_fx<NDET>(T, fx[p], sc, c * 32 + lane, C * 32, zh, zl);
+        warp_sums_df_to<NDET>(zh, zl, red[p][c], T.fxs);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const int p = lane / NDET, dd = lane - p * NDET;
+        double v = 0.0;
+        if (p < np) {
+            double zr = red[p][0][2 * dd], zi = red[p][0][2 * dd + 1];
+            for (int c = 1; c < C; c++) { zr += red[p][c][2 * dd]; zi += red[p][c][2 * dd + 1]; }
+            v = coef[p].gre[dd] * zr - coef[p].gim[dd] * zi;
+        }
+        const double t = group_sum_down<NDET>(v);
+        if (p < np && dd == 0) logl[i0 + p] = t - 0.5 * coef[p].hh;
+        if (st && lane == 0) {
+            unsigned long long n = 0;
+            for (int q = 0; q < np; q++) n += (unsigned long long)(coef[q].jcut + 1);
+            atomicAdd(&st->eval_points, (unsigned long long)np);
+            atomicAdd(&st->eval_point_bins, n);
+        }
+    }
+}
+
 template <int PREC, int NDET>
 cudaError_t eval_launch(const Model &M, const Tables &T, int warps, const double *in, int th, int m,
                         double *logl, RunState *st, cudaStream_t s) {
@@ -280,6 +342,15 @@ cudaError_t eval_launch(const Model &M, const Tables &T, int warps, const double
                 case 4: k_eval_batch<NDET, 4><<<gb, 128, 0, s>>>(M, T, in, m, logl, st); break;
                 default: k_eval_batch<NDET, 8><<<gb, 256, 0, s>>>(M, T, in, m, logl, st); break;
             }
+            return cudaGetLastError();
+        }
+    }
+    if constexpr (PREC == 0) {
+        if (M.model == M_GW && !th && !M.rb) {
+            // as many points a CTA as leave a CTA for every SM
+            int P = 1;
+            while (P < EVAL_FX_P && m >= 2 * P * 152) P *= 2;
+            k_eval_fx<NDET><<<(m + P - 1) / P, EVAL_FX_W * 32, 0, s>>>(M, T, in, m, P, warps, logl, st);
             return cudaGetLastError();
         }
     }
@@ -1050,7 +1121,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             const int wpc = 1 << lg, cand = warp >> lg, sub = warp & (wpc - 1);
             if (cand < ns) {
                 float zh[NDET][2], zl[NDET][2];
-                bins_fx<NDET>(T, fx[cand], sct, sub * 32 + lane, wpc * 32, coef[cand].jcut, zh, zl);
+                bins_fx<NDET>(T, fx[cand], sct, sub * 32 + lane, wpc * 32, zh, zl);
                 warp_sums_df_to<NDET>(zh, zl, &part[warp][0][0][0], T.fxs);
             }
             __syncthreads();
@@ -1075,7 +1146,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             if (PREC == 0) {
                 if (use_fx) {
                     float zh[NDET][2], zl[NDET][2];
-                    bins_fx<NDET>(T, fx[warp], sct, lane, 32, coef[warp].jcut, zh, zl);
+                    bins_fx<NDET>(T, fx[warp], sct, lane, 32, zh, zl);
                     v = warp_detector_terms_df<NDET>(zh, zl, coef[warp], T.fxs);
                 }
             } else if (M.tlg) {

@@ -52,6 +52,16 @@ int main() {
             for (int i = 0; i < 9; i++)
                 fx_mac(hi, cr, fx_split(fx_scaled(m[i], E - (ex[i] + 64) + 6, a[i])), fx_table(b[i], eb[i]));
             printf("%llu %d %d\n", (unsigned long long)fx_phase(hi, cr, E + 7), E, bad);
+        } else if (op[0] == 's') {
+            // levels, first bins, rows, bins to cover
+            FxTiles T;
+            FxPoint o;
+            T.nlev = (int)rd();
+            for (int i = 0; i < T.nlev; i++) { T.first[i] = (int)rd(); T.row[i] = (int)rd(); }
+            fx_segments(T, true, (int)rd(), o);
+            printf("%d %d", o.nseg, o.rows);
+            for (int i = 0; i < o.nseg; i++) printf(" %d %d", o.seg[i].end, o.seg[i].off);
+            printf("\n");
         } else {
             // n products w E summed
             float zh[2] = {0, 0}, zl[2] = {0, 0};
@@ -158,3 +168,34 @@ def test_products(fx):
         im = sum(mp.mpf(a) * mp.mpf(d) + mp.mpf(b) * mp.mpf(c) for a, b, c, d in v)
         size = sum(abs(a) + abs(b) for a, b, _, _ in v)
         assert abs(hexsum(t, 0) - re) <= size * 2.0 ** -46 and abs(hexsum(t, 2) - im) <= size * 2.0 ** -46
+
+
+@pytest.mark.parametrize("first", [[], [0], [128], [64, 256], [64, 128, 256, 1024], [0, 0, 0, 0, 0, 0, 0, 0, 0, 0],
+                                   [192, 256, 256, 512, 1024, 2048, 4096, 8192, 16384, 32768]])
+def test_segments(fx, first):
+    """The segments of every bin count cover each bin once, in order, by whole tiles of a level past its first bin."""
+    n = 70000 if len(first) == 10 else 9000
+    row, start = [], n
+    for l, f in enumerate(first):
+        row.append(start)
+        start += ((n - f) >> (6 + l)) * 32
+    head = f"s {len(first)} " + " ".join(f"{a} {b}" for a, b in zip(first, row)) + " "
+    rng = random.Random(1)
+    counts = sorted({0, 1, 63, 64, 65, n} | {rng.randrange(n + 1) for _ in range(400)}
+                    | {m + o for m in range(64, n, 64) for o in (0, 1) if rng.random() < 0.2})
+    for c, o in zip(counts, fx([head + str(c) for c in counts])):
+        v = list(map(int, o.split()))
+        segs, pos, r = list(zip(v[2::2], v[3::2])), 0, 0
+        assert v[0] == len(segs) <= 21
+        for end, off in segs:
+            lo = r + off
+            if lo < n:              # bins
+                assert lo == pos and lo + end - r <= n
+                pos += end - r
+            else:
+                l = max(i for i in range(len(first)) if row[i] <= lo and (i + 1 == len(first) or lo < row[i + 1]))
+                assert pos % (64 << l) == 0 and (lo - row[l]) == (pos - first[l]) // (64 << l) * 32 and pos >= first[l]
+                assert (end - r) % 32 == 0
+                pos += (end - r) // 32 * (64 << l)
+            r = end
+        assert pos == c and r == v[1]
