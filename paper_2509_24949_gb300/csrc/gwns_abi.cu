@@ -129,6 +129,21 @@ int capture_iteration(ns_ctx *c, int k) {
     return NS_OK;
 }
 
+// The binary exponents that bring the basis functions and the frequency below
+// one on the grid: each is monotone there but f^(1/3) ln f, whose minimum is -3/e
+// at f = e^-3.
+void fx_exponents(ns_ctx *c) {
+    const Model &M = c->M;
+    double mx[NB + 1] = {};
+    for (const double f : {M.f0, M.f0 + (double)(M.N - 1) * M.df}) {
+        const double r = std::cbrt(f), l = std::log(f);
+        const double B[NB + 1] = {1.0 / (f * r * r), 1.0 / f, 1.0 / (r * r), 1.0 / r, l, r, r * l, r * r, f};
+        for (int m = 0; m <= NB; m++) mx[m] = std::max(mx[m], std::fabs(B[m]));
+    }
+    mx[6] = std::max(mx[6], 1.2);
+    for (int m = 0; m <= NB; m++) c->T.fxe[m] = std::ilogb(std::max(mx[m] * (1.0 + 1e-12), 1e-300)) + 1;
+}
+
 // Relative-binning tables for the current data (edges, fiducial coefficients,
 // summary data); allocates on first use.
 int build_rb(ns_ctx *c) {
@@ -145,6 +160,12 @@ int build_rb(ns_ctx *c) {
             (rc = dalloc(&c->rb_A0f, nd * nb)) || (rc = dalloc(&c->rb_A1f, nd * nb)) ||
             (rc = dalloc(&c->rb_B0f, nd * nb)) || (rc = dalloc(&c->rb_B1f, nd * nb)) ||
             (rc = dalloc(&c->rb_inv_de_f, nb)))
+            return rc;
+        gwns::RBFx &X = c->rb_fx;
+        if (c->precision == NS_FP64 &&
+            ((rc = dalloc(&X.b, NB / 2 * ne)) || (rc = dalloc(&X.f, ne)) || (rc = dalloc(&X.G, nd * ne)) ||
+             (rc = dalloc(&X.GR, nd * ne)) || (rc = dalloc(&X.B, nd * nb)) || (rc = dalloc(&X.ys, nd)) ||
+             (rc = dalloc(&X.hs, nd)) || (rc = dalloc(&c->fx.sc, gwns::FX_SC))))
             return rc;
     }
     double2 *h0 = nullptr;
@@ -173,6 +194,14 @@ int build_rb(ns_ctx *c) {
     T.fm = c->rb_fm; T.inv_de = c->rb_inv_de; T.A0 = c->rb_A0; T.A1 = c->rb_A1; T.B0 = c->rb_B0;
     T.B1 = c->rb_B1; T.A0f = c->rb_A0f; T.A1f = c->rb_A1f; T.B0f = c->rb_B0f; T.B1f = c->rb_B1f;
     T.inv_de_f = c->rb_inv_de_f; T.fid = c->rb_fid;
+    if (c->precision == NS_FP64) {
+        const gwns::RBFx &X = c->rb_fx;
+        fx_exponents(c);
+        CK(gwns::launch_fx_sc(c->fx.sc, c->stream));
+        CK(gwns::launch_rb_fx(c->M, c->T, T, X, c->stream));
+        c->T.fxsc = c->fx.sc;
+        T.fxb = X.b; T.fxf = X.f; T.G = X.G; T.GR = X.GR; T.fxB = X.B; T.ys = X.ys; T.hs = X.hs;
+    }
     c->M.rb = 1;
     if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; c->graph_k = -1; }
     return NS_OK;
@@ -319,7 +348,8 @@ void ns_free(ns_ctx *c) {
     for (cudaEvent_t e : c->ev)
         if (e) cudaEventDestroy(e);
     void *bufs[] = {c->d_re, c->d_im, c->d_psd, c->basis64, c->f64, c->prefix, c->w64, c->fx.b, c->fx.f, c->fx.w, c->fx.scale,
-                    c->fx.sc, c->fx.wmax, c->fx.lag0, c->fx.lag1, c->fx.v[0], c->fx.v[1], c->X.basis32,
+                    c->fx.sc, c->fx.wmax, c->fx.lag0, c->fx.lag1, c->fx.v[0], c->fx.v[1], c->rb_fx.b, c->rb_fx.f,
+                    c->rb_fx.G, c->rb_fx.GR, c->rb_fx.B, c->rb_fx.ys, c->rb_fx.hs, c->X.basis32,
                     c->X.f32, c->X.w32, c->X.tb0, c->X.tb1, c->X.tbk, c->X.fc, c->X.wt, c->live_u, c->live_logl, c->order, c->chol, c->dead_u,
                     c->dead_logl, c->dead_logw, c->dead_nlive, c->state, c->scratch, c->fin_u,
                     c->fin_logl, c->fin_logw, c->fin_nlive, c->res, c->rb_J, c->rb_nedge, c->rb_fid,
@@ -489,8 +519,7 @@ static double tile_bound(const double *r, double fc, double h) {
 // prior draws (with 2% to spare; a point outside it is summed bin by bin), for
 // each tile length the first bin from which the bound above stays below 1e-15
 // (it falls with frequency, hence the bisection), and the matrices. Taken where
-// the draws' mean row count falls by a third or more, which leaves short segments
-// (4017 bins: 30 tiles or so over all draws) to the bins. GB300, batched
+// the draws' mean row count falls by a third or more. GB300, batched
 // likelihood of 2048 draws: 519,169 bins 15.3 ms -> 0.57 ms, 64,897 bins 169 -> 94 us.
 static int choose_tiles_fx(ns_ctx *c) {
     const Model &M = c->M;
@@ -606,20 +635,11 @@ static int choose_tiles_fx(ns_ctx *c) {
 }
 
 // FP64 form: the split tables (after the grid's FP64 tables are built: the tiles
-// are chosen from prior draws), and the binary exponents that bring the basis functions and
-// the frequency below one: each is monotone on the grid but f^(1/3) ln f, whose
-// minimum is -3/e at f = e^-3.
+// are chosen from prior draws).
 static int alloc_fx(ns_ctx *c) {
     const Model &M = c->M;
     const size_t nd = M.n_det;
-    double mx[NB + 1] = {};
-    for (const double f : {M.f0, M.f0 + (double)(M.N - 1) * M.df}) {
-        const double r = std::cbrt(f), l = std::log(f);
-        const double B[NB + 1] = {1.0 / (f * r * r), 1.0 / f, 1.0 / (r * r), 1.0 / r, l, r, r * l, r * r, f};
-        for (int m = 0; m <= NB; m++) mx[m] = std::max(mx[m], std::fabs(B[m]));
-    }
-    mx[6] = std::max(mx[6], 1.2);
-    for (int m = 0; m <= NB; m++) c->T.fxe[m] = std::ilogb(std::max(mx[m] * (1.0 + 1e-12), 1e-300)) + 1;
+    fx_exponents(c);
     c->fx.n = M.N;
     int rc = choose_tiles_fx(c);
     if (rc) return rc;
@@ -806,7 +826,8 @@ int ns_init(ns_ctx **out, const ns_prior *prior, const ns_data *data, const ns_p
         if (e == cudaSuccess) e = build_tables(c);
         if (e == cudaSuccess && split) {
             if ((rc = alloc_fx(c))) { ns_free(c); return rc; }
-            e = launch_build_fx(c->M, c->T, c->w64, c->fx, c->stream);
+            e = gwns::launch_fx_sc(c->fx.sc, c->stream);
+            if (e == cudaSuccess) e = launch_build_fx(c->M, c->T, c->w64, c->fx, c->stream);
         }
     }
     if (e != cudaSuccess) { ns_free(c); return cuda_fail(e); }

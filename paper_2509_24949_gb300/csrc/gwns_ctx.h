@@ -62,6 +62,7 @@ struct ns_ctx {
     double *rb_B0 = nullptr, *rb_B1 = nullptr;
     double2 *rb_A0 = nullptr, *rb_A1 = nullptr;
     float2 *rb_basis32 = nullptr, *rb_fe32 = nullptr, *rb_A0f = nullptr, *rb_A1f = nullptr;
+    gwns::RBFx rb_fx = {};           // FP64 form
     float *rb_B0f = nullptr, *rb_B1f = nullptr, *rb_inv_de_f = nullptr;
     // result buffers
     double *fin_u = nullptr, *fin_logl = nullptr, *fin_logw = nullptr, *fin_nlive = nullptr;

@@ -83,6 +83,14 @@ struct RBTables {
     const float2 *A0f, *A1f;   // FP32 copies for the mixed form
     const float *B0f, *B1f, *inv_de_f;
     const Coef *fid;           // fiducial point's coefficients
+    // FP64 form (gwns_fx.cuh): the edges' basis and frequency; the edges' summary
+    // coefficients G (both neighbouring bins) and GR (the lower bin only) over the
+    // scale ys[d], and the bins' B0 over hs[d], in double-float
+    const int4 *fxb;           // [NB/2][nedge]
+    const int2 *fxf;           // [nedge]
+    const float4 *G, *GR;      // [n_det][nedge]
+    const float2 *fxB;         // [n_det][nb]
+    const double *ys, *hs;     // [n_det]
 };
 
 // Device tables of one grid.
@@ -793,7 +801,9 @@ __device__ __forceinline__ void sincos_bf(double x, double &s, double &c) {
 // one scale per point (gwns_fx.cuh): lane group g (8 lanes) takes point g, its
 // sub-lane m basis coefficient m, then detector m's delay and (sub-lane 0) the
 // constant phase. Integer instructions only. All 32 lanes must call.
-__device__ inline void coef_to_fx_group(const Tables &T, int n_det, const Coef *c0, FxPoint *out0, int count) {
+// With fid, the differences from the fiducial point's coefficients.
+__device__ inline void coef_to_fx_group(const Tables &T, int n_det, const Coef *c0, FxPoint *out0, int count,
+                                        const Coef *fid = nullptr) {
     const int lane = threadIdx.x & 31, g = lane >> 3, sl = lane & 7;
     const bool writer = g < count;
     const Coef &c = c0[writer ? g : 0];
@@ -801,7 +811,12 @@ __device__ inline void coef_to_fx_group(const Tables &T, int n_det, const Coef *
     int bad = 0;
     uint64_t ma, mt, mc;
     const bool det = sl < n_det;
-    const double a = c.a[sl], tau = c.tau[det ? sl : 0], ph = c.c0u;
+    double a = c.a[sl], tau = c.tau[det ? sl : 0], ph = c.c0u;
+    if (fid) {
+        a -= fid->a[sl];
+        tau -= fid->tau[det ? sl : 0];
+        ph -= fid->c0u;
+    }
     const int ea = fx_mantissa<true>(a, &ma, &bad) + T.fxe[sl];
     const int et = fx_mantissa<false>(tau, &mt, &bad) + T.fxe[NB];
     const int ec = fx_mantissa<true>(ph, &mc, &bad);
@@ -1591,48 +1606,90 @@ __device__ __forceinline__ void warp_sum_df_many(float (&h)[16], float (&l)[16],
 // so that with rho_d = conj(G_d)/conj(G0_d) (r = h/h0 = rho_d E_d):
 //   <d|h_d> = Re(conj(rho_d) Y_d),  <h_d|h_d> = |rho_d|^2 H_d.
 // Bins whose centre lies above f_ISCO are dropped when the cutoff is on.
+//
+// FP64 form. With C_e = conj(E(e)) the sums over bins are
+//   Y_d = sum_e G_e C_e,  G_e = (A0_e/2 - A1_e/de_e) + (A0_e-1/2 + A1_e-1/de_e-1),
+//   H_d = sum_b B0_b (1 + Re(C_b conj C_b+1))/2
+// (|C| = 1, so |S|^2/4 = (1 + Re ..)/2 and the B1 term vanishes); at the last used
+// edge G is its lower bin's part alone (GR). One warp, 31 bins a pass, in the
+// split arithmetic of gwns_fx.cuh: about 600 cycles a pass and three detectors,
+// against 11,000 for the FP64 sines, cosines and sums. GB300, 8192 draws on 1024
+// coarse bins: 2.81 ms -> 237 us.
 template <int NDET>
-__device__ __forceinline__ void rb_fp64(const Model &M, const RBTables &R, const Coef &c, int lane,
-                                        double Yr[NDET], double Yi[NDET], double H[NDET]) {
-    const Coef &f = *R.fid;
-    double da[NB];
-#pragma unroll
-    for (int m = 0; m < NB; m++) da[m] = c.a[m] - f.a[m];
-    const double dc = c.c0 - f.c0;
-    double dtau[NDET];
-#pragma unroll
-    for (int d = 0; d < NDET; d++) { dtau[d] = c.tau[d] - f.tau[d]; Yr[d] = Yi[d] = H[d] = 0.0; }
-    for (int base = 0; base < R.nb; base += 31) {
-        const int e = base + lane;
-        const bool ok = e < R.nedge;
-        double psi = dc;
-        if (ok) {
-#pragma unroll
-            for (int m = 0; m < NB; m++) psi = fma(da[m], __ldg(R.basis64 + (size_t)m * R.nedge + e), psi);
+__device__ __forceinline__ double rb_loglike_fx(const Model &M, const RBTables &R, const Coef &c, const FxPoint &fx,
+                                                const float4 *sc) {
+    const int lane = threadIdx.x & 31;
+    // bins whose centre lies at or below f_ISCO: a 32-way search (the centres ascend)
+    int nbu = R.nb;
+    if (M.cutoff) {
+        int lo = 0, hi = R.nb;
+        while (hi > lo) {
+            const int step = (hi - lo + 31) >> 5, i = lo + lane * step;
+            const int n = __popc(__ballot_sync(0xffffffffu, i < hi && __ldg(R.fm + i) <= c.fisco));
+            if (n == 0) break;
+            const int next = lo + n * step;
+            lo = lo + (n - 1) * step + 1;
+            hi = min(hi, next);
         }
-        const double fe = ok ? __ldg(R.fe + e) : 0.0;
-        const int b = base + lane;
-        const bool use = lane < 31 && b < R.nb && (!M.cutoff || __ldg(R.fm + b) <= c.fisco);
+        nbu = lo;
+    }
+    float vh[16], vl[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        vh[i] = (fx.bad && nbu > 0) ? __int_as_float(0x7fffffff) : 0.f;
+        vl[i] = 0.f;
+    }
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int ne = R.nedge;
+#pragma unroll 1
+    for (int base = 0; base < nbu && !fx.bad; base += 31) {
+        const int e = min(base + lane, nbu);
+        const bool own = lane < 31 && base + lane < nbu, last = base + lane == nbu;
+        int64_t hi = fx.c0, cr = 0;
+#pragma unroll
+        for (int m = 0; m < NB; m += 2) {
+            const int4 b = __ldg(R.fxb + (size_t)(m >> 1) * ne + e);
+            fx_mac(hi, cr, fx.a[m], fx2{b.x, b.y});
+            fx_mac(hi, cr, fx.a[m + 1], fx2{b.z, b.w});
+        }
+        const int2 f = __ldg(R.fxf + e);
 #pragma unroll
         for (int d = 0; d < NDET; d++) {
-            double sn, cs;
-            sincos(psi + TWO_PI_D * fe * dtau[d], &sn, &cs);
-            const double er = cs, ei = -sn;                    // exp(-i dPsi)
-            const double nr = __shfl_down_sync(0xffffffffu, er, 1);
-            const double ni = __shfl_down_sync(0xffffffffu, ei, 1);
-            if (use) {
-                const double idl = __ldg(R.inv_de + b);
-                const double Sr = er + nr, Si = ei + ni;
-                const double Dr = (nr - er) * idl, Di = (ni - ei) * idl;
-                const size_t o = (size_t)d * R.nb + b;
-                const double2 a0 = __ldg(R.A0 + o), a1 = __ldg(R.A1 + o);
-                // A0 conj(S)/2 + A1 conj(D)
-                Yr[d] += 0.5 * (a0.x * Sr + a0.y * Si) + (a1.x * Dr + a1.y * Di);
-                Yi[d] += 0.5 * (a0.y * Sr - a0.x * Si) + (a1.y * Dr - a1.x * Di);
-                H[d] += 0.25 * __ldg(R.B0 + o) * (Sr * Sr + Si * Si) + __ldg(R.B1 + o) * (Sr * Dr + Si * Di);
-            }
+            int64_t hd = hi, cd = cr;
+            fx_mac(hd, cd, fx.t[d], fx2{f.x, f.y});
+            const fxe E = fx_cis(fx_phase(hd, cd, fx.sh), sc);
+            const float4 *gp = (last ? R.GR : R.G) + (size_t)d * ne + e;
+            const float4 w = own || last ? __ldg(gp) : zero;
+            fx_acc(vh[3 * d], vl[3 * d], w.x, w.y, E.rh, E.rl);
+            fx_acc(vh[3 * d], vl[3 * d], -w.z, -w.w, E.ih, E.il);
+            fx_acc(vh[3 * d + 1], vl[3 * d + 1], w.x, w.y, E.ih, E.il);
+            fx_acc(vh[3 * d + 1], vl[3 * d + 1], w.z, w.w, E.rh, E.rl);
+            // Re(C_b conj C_b+1) from the next lane's edge
+            const float nrh = __shfl_down_sync(0xffffffffu, E.rh, 1), nrl = __shfl_down_sync(0xffffffffu, E.rl, 1);
+            const float nih = __shfl_down_sync(0xffffffffu, E.ih, 1), nil = __shfl_down_sync(0xffffffffu, E.il, 1);
+            const float p = f_mul(E.rh, nrh), q = f_mul(E.ih, nih);
+            float pe = f_fma(E.rh, nrh, -p), qe = f_fma(E.ih, nih, -q);
+            pe = f_fma(E.rl, nrh, f_fma(E.rh, nrl, pe));
+            qe = f_fma(E.il, nih, f_fma(E.ih, nil, qe));
+            const dfl s = two_sum_f(p, q), t = fast_two_sum_f(1.0f, s.h);
+            const float2 b0 = own ? __ldg(R.fxB + (size_t)d * R.nb + e) : make_float2(0.f, 0.f);
+            fx_acc(vh[3 * d + 2], vl[3 * d + 2], b0.x, b0.y, 0.5f * t.h, 0.5f * (t.l + (s.l + (pe + qe))));
         }
     }
+    float rh, rl;
+    warp_sum_df_many<3 * NDET>(vh, vl, rh, rl);
+    // lane d forms detector d's terms: lanes 2v hold value v = 3 d + (Re Y, Im Y, H)
+    const int d = min(lane, NDET - 1);
+    const double z = (double)rh + (double)rl;
+    const double yr = __shfl_sync(0xffffffffu, z, 6 * d) * __ldg(R.ys + d);
+    const double yi = __shfl_sync(0xffffffffu, z, 6 * d + 2) * __ldg(R.ys + d);
+    const double h = __shfl_sync(0xffffffffu, z, 6 * d + 4) * __ldg(R.hs + d);
+    // rho = conj(G)/conj(G0)
+    const double g0r = R.fid->gre[d], g0i = R.fid->gim[d];
+    const double den = g0r * g0r + g0i * g0i;
+    const double rr = (c.gre[d] * g0r + c.gim[d] * g0i) / den;
+    const double ri = -(c.gim[d] * g0r - c.gre[d] * g0i) / den;
+    return group_sum_down<NDET>((rr * yr + ri * yi) - 0.5 * (rr * rr + ri * ri) * h);
 }
 
 template <int NDET>
@@ -1694,13 +1751,12 @@ __device__ __forceinline__ void rb_mixed(const Model &M, const RBTables &R, cons
     for (int d = 0; d < NDET; d++) { Yr[d] = yr[d]; Yi[d] = yi[d]; H[d] = hh[d]; }
 }
 
-// log L of one point from the relative-binning sums (lane 0 holds the result).
-template <int NDET, int PREC>
-__device__ __forceinline__ double rb_loglike_warp(const Model &M, const RBTables &R, const Coef &c,
-                                                  const CoefMixed &cm, int lane) {
+// Mixed form: log L of one point from the relative-binning sums (lane 0 holds the result).
+template <int NDET>
+__device__ __forceinline__ double rb_loglike_mixed(const Model &M, const RBTables &R, const Coef &c,
+                                                   const CoefMixed &cm, int lane) {
     double Yr[NDET], Yi[NDET], H[NDET];
-    if (PREC == 0) rb_fp64<NDET>(M, R, c, lane, Yr, Yi, H);
-    else rb_mixed<NDET>(M, R, cm, c.fisco, lane, Yr, Yi, H);
+    rb_mixed<NDET>(M, R, cm, c.fisco, lane, Yr, Yi, H);
     double v = 0.0;
 #pragma unroll
     for (int d = 0; d < NDET; d++) {

@@ -244,16 +244,23 @@ __device__ __forceinline__ float2 fx_df(double x) {
     return make_float2(h, isfinite(h) ? __double2float_rn(x - (double)h) : 0.f);
 }
 
+__global__ void k_fx_sc(float4 *sc) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= FX_SC) return;
+    double sn, cs;
+    sincospi((double)i * (1.0 / FX_SC), &sn, &cs);
+    const float2 c = fx_df(cs), s = fx_df(sn);
+    sc[i] = make_float4(c.x, c.y, s.x, s.y);
+}
+cudaError_t launch_fx_sc(float4 *sc, cudaStream_t s) {
+    k_fx_sc<<<(FX_SC + 127) / 128, 128, 0, s>>>(sc);
+    return cudaGetLastError();
+}
+
 // .. and the tables: fixed-point basis and frequency, the data scaled by the
 // power of two that takes the detector's largest |w| into [1, 2).
 __global__ void k_build_fx(Model M, Tables T, const double2 *w64, FxTables X) {
     const int i0 = blockIdx.x * blockDim.x + threadIdx.x, st = gridDim.x * blockDim.x;
-    for (int i = i0; i < FX_SC; i += st) {
-        double sn, cs;
-        sincospi((double)i * (1.0 / FX_SC), &sn, &cs);
-        const float2 c = fx_df(cs), s = fx_df(sn);
-        X.sc[i] = make_float4(c.x, c.y, s.x, s.y);
-    }
     int e[MAXDET];
 #pragma unroll
     for (int d = 0; d < MAXDET; d++) {
@@ -384,7 +391,7 @@ cudaError_t launch_build_fx(const Model &M, const Tables &T, const double2 *w64,
     if (e != cudaSuccess) return e;
     const int blocks = min((M.N + 255) / 256, 152 * 4);
     k_fx_wmax<<<dim3(blocks, M.n_det), 256, 0, s>>>(w64, M.N, M.n_det, X.wmax);
-    k_build_fx<<<min((max(M.N, FX_SC) + 127) / 128, 152 * 8), 128, 0, s>>>(M, T, w64, X);
+    k_build_fx<<<min((M.N + 127) / 128, 152 * 8), 128, 0, s>>>(M, T, w64, X);
     for (int l = 0; l < T.tiles.nlev; l++) {
         const int tiles = (M.N - T.tiles.first[l]) >> (FX_LG0 + l);
         k_fx_nodes<<<tiles, 32 * M.n_det, 0, s>>>(M, T, w64, X, l, X.v[(l + 1) & 1], X.v[l & 1]);
@@ -1007,6 +1014,66 @@ cudaError_t launch_rb_setup(const Model &M, const Tables &T, int B, const double
     dim3 grid(B, M.n_det);
     k_rb_summary<<<grid, 256, 0, s>>>(M, J, nedge_dev, dre, dim, psd, h0_tmp, R, fe, basis64, basis32, fe32,
                                       fm, inv_de, A0, A1, B0, B1, A0f, A1f, B0f, B1f, inv_de_f);
+    return cudaGetLastError();
+}
+
+// FP64 form's split tables of the summary data, one CTA: the edges' coefficients
+// G_e and GR_e and the bins' B0, each over the power of two of the detector's
+// largest, and the edges' fixed-point basis and frequency.
+__global__ void __launch_bounds__(1024) k_rb_fx(int nd, Tables T, RBTables R, RBFx X) {
+    __shared__ unsigned mx[2][MAXDET];
+    const int ne = R.nedge, nb = R.nb;
+    if (threadIdx.x < 2 * MAXDET) ((unsigned *)mx)[threadIdx.x] = 0;
+    __syncthreads();
+    auto part = [&](int d, int b, double sign) {        // A0/2 + sign A1/de of bin b (0 outside)
+        if (b < 0 || b >= nb) return make_double2(0.0, 0.0);
+        const double2 a0 = R.A0[(size_t)d * nb + b], a1 = R.A1[(size_t)d * nb + b];
+        const double k = sign * R.inv_de[b];
+        return make_double2(0.5 * a0.x + k * a1.x, 0.5 * a0.y + k * a1.y);
+    };
+    auto mag = [](double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; };
+    for (int d = 0; d < nd; d++) {
+        unsigned y = 0, h = 0;
+        for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+            const double2 r = part(d, e - 1, 1.0), l = part(d, e, -1.0);
+            y = max(y, max(max(mag(r.x), mag(r.y)), max(mag(r.x + l.x), mag(r.y + l.y))));
+            if (e < nb) h = max(h, mag(R.B0[(size_t)d * nb + e]));
+        }
+        atomicMax(&mx[0][d], y);
+        atomicMax(&mx[1][d], h);
+    }
+    __syncthreads();
+    for (int d = 0; d < nd; d++) {
+        const int xy = (int)(mx[0][d] >> 20), xh = (int)(mx[1][d] >> 20);
+        const int ey = (xy == 0 || xy == 0x7ff) ? 0 : xy - 1023, eh = (xh == 0 || xh == 0x7ff) ? 0 : xh - 1023;
+        if (threadIdx.x == 0) {
+            X.ys[d] = scalbn(1.0, ey);
+            X.hs[d] = scalbn(1.0, eh);
+        }
+        for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+            const double2 r = part(d, e - 1, 1.0), l = part(d, e, -1.0);
+            const size_t o = (size_t)d * ne + e;
+            float2 re = fx_df(scalbn(r.x, -ey)), im = fx_df(scalbn(r.y, -ey));
+            X.GR[o] = make_float4(re.x, re.y, im.x, im.y);
+            re = fx_df(scalbn(r.x + l.x, -ey));
+            im = fx_df(scalbn(r.y + l.y, -ey));
+            X.G[o] = make_float4(re.x, re.y, im.x, im.y);
+            if (e < nb) X.B[(size_t)d * nb + e] = fx_df(scalbn(R.B0[(size_t)d * nb + e], -eh));
+        }
+    }
+    for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+        for (int m = 0; m < NB; m += 2) {
+            const fx2 a = fx_table(R.basis64[(size_t)m * ne + e], T.fxe[m]);
+            const fx2 b = fx_table(R.basis64[(size_t)(m + 1) * ne + e], T.fxe[m + 1]);
+            X.b[(size_t)(m >> 1) * ne + e] = make_int4(a.h, a.l, b.h, b.l);
+        }
+        const fx2 f = fx_table(R.fe[e], T.fxe[NB]);
+        X.f[e] = make_int2(f.h, f.l);
+    }
+}
+
+cudaError_t launch_rb_fx(const Model &M, const Tables &T, const RBTables &R, const RBFx &X, cudaStream_t s) {
+    k_rb_fx<<<1, 1024, 0, s>>>(M.n_det, T, R, X);
     return cudaGetLastError();
 }
 

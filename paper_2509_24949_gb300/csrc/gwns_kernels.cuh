@@ -159,6 +159,17 @@ cudaError_t launch_build_tables(const Model &M, const double *data_re, const dou
                                 const double *psd, double *basis64, double *f64, double2 *w64,
                                 double *prefix, const MixedTables &X, cudaStream_t s);
 // The FP64 form's split tables from the grid's basis64, f64 and w64 (exponents: Tables::fxe).
+// The cosine and sine table (Tables::fxsc).
+cudaError_t launch_fx_sc(float4 *sc, cudaStream_t s);
+// Relative binning, FP64 form: the split tables from the summary data (RBTables, writable here).
+struct RBFx {
+    int4 *b;
+    int2 *f;
+    float4 *G, *GR;
+    float2 *B;
+    double *ys, *hs;
+};
+cudaError_t launch_rb_fx(const Model &M, const Tables &T, const RBTables &R, const RBFx &X, cudaStream_t s);
 // Phase coefficients of m prior draws (the first 16 at the corners of the mass and spin ranges).
 cudaError_t launch_prior_coefs(const Model &M, const Tables &T, int m, Coef *out, cudaStream_t s);
 cudaError_t launch_build_fx(const Model &M, const Tables &T, const double2 *w64, const FxTables &X, cudaStream_t s);

@@ -121,7 +121,7 @@ __device__ __forceinline__ void warp_point_coef(const Model &M, const Tables &T,
     }
     __syncwarp();
     if (precision == 1) coef_to_mixed_warp(*coef, M.n_det, M.df, cm, M.rb ? T.rb.fid : nullptr, M.tlg >= 5);
-    else if (!M.rb) coef_to_fx_group(T, M.n_det, coef, fx, 1);
+    else coef_to_fx_group(T, M.n_det, coef, fx, 1, M.rb ? T.rb.fid : nullptr);
 }
 
 // Points per CTA of the batched likelihood: the coefficient stage packs up to
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(W * 32) k_eval(Model M, Tables T, const double
     __shared__ float4 sc[PREC == 0 ? FX_SC : 1];
     const int i0 = blockIdx.x * ppc;
     if (i0 >= m) return;
-    if (PREC == 0 && M.model == M_GW && !M.rb) load_sc(T, sc);
+    if (PREC == 0 && M.model == M_GW) load_sc(T, sc);
     const int np = m - i0 < ppc ? m - i0 : ppc;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stride_in = in_is_theta ? NPARAM : M.dim;
@@ -167,7 +167,8 @@ __global__ void __launch_bounds__(W * 32) k_eval(Model M, Tables T, const double
         if (M.rb) {
             // relative-binning sums: one warp
             if (warp == 0) {
-                const double v = rb_loglike_warp<NDET, PREC>(M, T.rb, coef[p], cm[p], lane);
+                const double v = PREC == 0 ? rb_loglike_fx<NDET>(M, T.rb, coef[p], fx, sc)
+                                           : rb_loglike_mixed<NDET>(M, T.rb, coef[p], cm[p], lane);
                 if (lane == 0) {
                     logl[i0 + p] = v;
                     if (st) atomicAdd(&st->eval_points, 1ull);
@@ -278,7 +279,8 @@ __global__ void __launch_bounds__(W * 32) k_eval_batch(Model M, Tables T, const 
 constexpr int EVAL_FX_W = 4;                // warps
 constexpr int EVAL_FX_P = EVAL_FX_W;        // points at most
 
-template <int NDET>
+// Relative binning (RB): one warp sums a point's coarse bins (C = 1).
+template <int NDET, bool RB>
 __global__ void __launch_bounds__(EVAL_FX_W * 32, 16 / EVAL_FX_W) k_eval_fx(Model M, Tables T, const double *in,
                                                                             int m, int P, int C, double *logl,
                                                                             RunState *st) {
@@ -298,10 +300,18 @@ __global__ void __launch_bounds__(EVAL_FX_W * 32, 16 / EVAL_FX_W) k_eval_fx(Mode
     if (cnt > 0) point_coef_group(M, T, pt[4 * grp], MAXD, &coef[4 * grp], cnt, 1 + (warp & 1));
     __syncthreads();
     if (cnt > 0) {
-        if (warp & 1) coef_to_fx_group(T, M.n_det, &coef[4 * grp], &fx[4 * grp], cnt);
+        if (warp & 1) coef_to_fx_group(T, M.n_det, &coef[4 * grp], &fx[4 * grp], cnt, RB ? T.rb.fid : nullptr);
         else point_coef_join(M, T, &coef[4 * grp], cnt);
     }
     __syncthreads();
+    if constexpr (RB) {
+        for (int p = warp; p < np; p += EVAL_FX_W) {
+            const double v = rb_loglike_fx<NDET>(M, T.rb, coef[p], fx[p], sc);
+            if (lane == 0) logl[i0 + p] = v;
+        }
+        if (st && threadIdx.x == 0) atomicAdd(&st->eval_points, (unsigned long long)np);
+        return;
+    }
     for (int it = warp; it < np * C; it += EVAL_FX_W) {
         const int p = it / C, c = it - p * C;
         float zh[NDET][2], zl[NDET][2];
@@ -346,11 +356,12 @@ cudaError_t eval_launch(const Model &M, const Tables &T, int warps, const double
         }
     }
     if constexpr (PREC == 0) {
-        if (M.model == M_GW && !th && !M.rb) {
+        if (M.model == M_GW && !th) {
             // as many points a CTA as leave a CTA for every SM
             int P = 1;
             while (P < EVAL_FX_P && m >= 2 * P * 152) P *= 2;
-            k_eval_fx<NDET><<<(m + P - 1) / P, EVAL_FX_W * 32, 0, s>>>(M, T, in, m, P, warps, logl, st);
+            if (M.rb) k_eval_fx<NDET, true><<<(m + P - 1) / P, EVAL_FX_W * 32, 0, s>>>(M, T, in, m, P, 1, logl, st);
+            else k_eval_fx<NDET, false><<<(m + P - 1) / P, EVAL_FX_W * 32, 0, s>>>(M, T, in, m, P, warps, logl, st);
             return cudaGetLastError();
         }
     }
@@ -926,7 +937,8 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
     __shared__ float4 sct[PREC == 0 ? FX_SC : 1];
     if (chain >= A.k) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d = M.dim;
-    const bool use_fx = PREC == 0 && M.model == M_GW && !M.rb;
+    const bool use_fx = PREC == 0 && M.model == M_GW;
+    const Coef *fid = M.rb ? T.rb.fid : nullptr;
     if (use_fx) load_sc(T, sct);    // used after the first round's barriers
     const uint32_t iter = (uint32_t)A.state->iter;
     const double lstar = A.state->lstar;
@@ -1014,7 +1026,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             if (warp == 0) point_coef_join(M, T, coef, ns);
             // meanwhile the odd warp of each group of four: the fixed-point coefficients
             if (use_fx && (warp & 1) && 4 * grp < ns)
-                coef_to_fx_group(T, M.n_det, &coef[4 * grp], &fx[4 * grp], min(4, ns - 4 * grp));
+                coef_to_fx_group(T, M.n_det, &coef[4 * grp], &fx[4 * grp], min(4, ns - 4 * grp), fid);
             __syncthreads();
         } else {
             if (4 * warp < ns) {
@@ -1026,18 +1038,21 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                     point_coef_group(M, T, ysh[4 * warp], MAXD, &coef[4 * warp], cnt);
                 if (use_fx) {
                     __syncwarp();
-                    coef_to_fx_group(T, M.n_det, &coef[4 * warp], &fx[4 * warp], cnt);
+                    coef_to_fx_group(T, M.n_det, &coef[4 * warp], &fx[4 * warp], cnt, fid);
                 }
             }
             __syncthreads();
         }
         if (warp < ns && M.rb) {
             // relative-binning likelihood of the slot's candidate
+            double v;
             if (PREC == 1) {
                 coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], T.rb.fid);
                 __syncwarp();
+                v = rb_loglike_mixed<NDET>(M, T.rb, coef[warp], cm[warp], lane);
+            } else {
+                v = rb_loglike_fx<NDET>(M, T.rb, coef[warp], fx[warp], sct);
             }
-            const double v = rb_loglike_warp<NDET, PREC>(M, T.rb, coef[warp], cm[warp], lane);
             if (lane == 0) {
                 lval[warp] = v;
                 coef[warp].jcut = T.rb.nb - 1;     // bins counted for the work statistics
@@ -1144,7 +1159,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             // one candidate per slot warp: bins and warp reduction
             double v = 0.0;
             if (PREC == 0) {
-                if (use_fx) {
+                if (M.model == M_GW) {
                     float zh[NDET][2], zl[NDET][2];
                     bins_fx<NDET>(T, fx[warp], sct, lane, 32, zh, zl);
                     v = warp_detector_terms_df<NDET>(zh, zl, coef[warp], T.fxs);

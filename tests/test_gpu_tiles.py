@@ -77,3 +77,14 @@ def test_batch_sizes_and_nan(gw):
         v[4, 7] = np.nan
         got = sp.eval_lnl(v)
     assert np.isnan(got[4]) and np.array_equal(np.delete(got, 4), np.delete(full[:9], 4))
+
+
+@pytest.mark.parametrize("bins", [1, 2, 30, 31, 32, 62, 63, 95, 700])
+@pytest.mark.parametrize("n_det", [1, 3, 4])
+def test_coarse_bin_counts(gw, bins, n_det):
+    """Passes of 31 coarse bins: counts about their multiples, cutoffs among them."""
+    w, pb, th = problem("c1", n_det=n_det)
+    rb = oracle.RelativeBinning(pb, th, B=bins)
+    u = pts_for(pb, th, count=33)
+    with sampler_from(gw, pb, 0, n_live=8, coarse_bins=bins, theta_fid=th) as sp:
+        assert close(sp.eval_lnl(u), rb.loglike(u))
