@@ -269,14 +269,25 @@ __device__ __forceinline__ void prior_transform(const Model &M, const double *u,
 // --------------------------------------------------------- point coefficients
 // Last grid index with f_j <= fisco, in [-1, N-1], from the grid's frequency
 // table (f64[j] holds the rounded f0 + j*df the tables use): a first guess by
-// one multiplication, then at most a few steps either way against the table.
+// one multiplication, then at most a few steps either way against the table. The
+// guess is in FP32 where that is within a bin or so, the comparisons are of the
+// bit patterns (positive doubles order as their bits do): FP64 instructions cost
+// 64 cycles each. A NaN or a fisco that is not positive gives -1.
 __device__ __forceinline__ int cutoff_index_tab(const Model &M, const double *f64, double fisco) {
     if (!M.cutoff) return M.N - 1;
-    const double jf = floor((fisco - M.f0) * M.inv_df);
-    if (!(jf >= -1.0)) return -1;
-    int j = jf > (double)(M.N - 1) ? M.N - 1 : (int)jf;
-    for (int it = 0; it < 4 && j + 1 <= M.N - 1 && __ldg(f64 + j + 1) <= fisco; it++) j++;
-    for (int it = 0; it < 4 && j >= 0 && __ldg(f64 + j) > fisco; it++) j--;
+    const long long fb = __double_as_longlong(fisco);
+    if (fb <= 0 || fb > 0x7ff0000000000000ll) return -1;
+    int j;
+    if (M.N <= (1 << 20)) {
+        const float g = ((float)fisco - (float)M.f0) * (float)M.inv_df;
+        j = g < -1.0f ? -1 : g > (float)(M.N - 1) ? M.N - 1 : (int)floorf(g);
+    } else {
+        const double jf = floor((fisco - M.f0) * M.inv_df);
+        j = jf < -1.0 ? -1 : jf > (double)(M.N - 1) ? M.N - 1 : (int)jf;
+    }
+    auto le = [&](int i) { return __double_as_longlong(__ldg(f64 + i)) <= fb; };
+    for (int it = 0; it < 8 && j + 1 <= M.N - 1 && le(j + 1); it++) j++;
+    for (int it = 0; it < 8 && j >= 0 && !le(j); it++) j--;
     return j;
 }
 
@@ -298,6 +309,16 @@ __device__ __forceinline__ int cutoff_index_tab(const Model &M, const double *f6
     F(PI_D * 77096675.0 / 254016.0), F(PI_D * 378515.0 / 1512.0), F(-PI_D * 74045.0 / 756.0), F(0.0)
 #define GWNS_AS_DOUBLE(x) (x)
 __device__ const double PN_POLY[NB * 4] = {GWNS_PN_POLY(GWNS_AS_DOUBLE)};
+// spin and log rows of the same coefficients (point_coef_group): s0 s1 s2, d0 d1, e, l
+__device__ const double PN_SPIN[NB * 8] = {
+    0, 0, 0, 0, 0, 0, 0, 0,
+    0, 0, 0, 0, 0, 0, 0, 0,
+    113.0 / 6.0, -38.0 / 3.0, 0, 113.0 / 6.0, 0, 0, 0, 0,
+    0, 0, 0, 0, 0, -395.0 / 4.0, 0, 0,
+    -732985.0 / 4536.0, 12130.0 / 81.0, 170.0 / 9.0, -732985.0 / 4536.0, -70.0 / 9.0, 0, 0, 0,
+    0, 0, 0, 0, 0, 0, -6848.0 / 21.0, 0,
+    0, 0, 0, 0, 0, 0, 0, 0,
+    0, 0, 0, 0, 0, 0, 0, 0};
 // the same as double-floats, for the mixed form's coefficient stage
 __device__ const dfl PN_POLY_X[NB * 4] = {GWNS_PN_POLY(DFC)};
 
@@ -318,43 +339,29 @@ __device__ inline void point_coef_group(const Model &M, const Tables &T, const d
     const bool writer = g < count;
     const double *u = u0 + (writer ? g : 0) * ustride;
     Coef *out = out0 + (writer ? g : 0);
-    // prior transform; a uniform-in-volume distance keeps its volume argument
-    double th[NPARAM];
-    double dl_arg = 0.0;
-    bool dl_vol = false;
-    {
-        int i = 0;
+    // prior transform: sub-lane s forms parameters s and s + 8; a uniform-in-volume
+    // distance keeps its volume argument
+    double thp[2];
 #pragma unroll
-        for (int p = 0; p < NPARAM; p++) {
-            // each half transforms only the parameters it uses (mass and phase:
-            // chirp mass, q, spins, distance, phi_c; sky and detectors: cos i,
-            // psi, t_c, RA, sin dec)
-            const bool mass_p = p == P_MC || p == P_Q || p == P_CHI1 || p == P_CHI2 || p == P_DL || p == P_PHIC;
-            if (M.kind[p] == K_FIXED) {
-                th[p] = M.lo[p];
-            } else if ((half == 1 && !mass_p) || (half == 2 && mass_p)) {
-                th[p] = 0.0;
-                i++;
-            } else if (M.kind[p] == K_UNIFORM) {
-                th[p] = fma(M.pspan[p], u[i++], M.pbase[p]);
-            } else {
-                const double v = fma(M.pspan[p], u[i++], M.pbase[p]);
-                if (p == P_DL) { dl_vol = true; dl_arg = v; th[p] = 0.0; }
-                else th[p] = cbrt(v);
-            }
-        }
-        if (!dl_vol) dl_arg = th[P_DL];
+    for (int r = 0; r < 2; r++) {
+        const int p = sl + 8 * r < NPARAM ? sl + 8 * r : 0;
+        const int kind = M.kind[p];
+        double v = M.lo[p];
+        if (kind != K_FIXED) v = fma(M.pspan[p], u[M.uidx[p]], M.pbase[p]);
+        if (kind == K_VOLUME && p != P_DL) v = cbrt(v);
+        thp[r] = v;
     }
+    auto TH = [&](int p) { return __shfl_sync(FULL, p < 8 ? thp[0] : thp[1], p & 7, 8); };
+    const bool dl_vol = M.kind[P_DL] == K_VOLUME;
     // mass and phase part (half 0 or 1)
     double amp = 0.0;
     int jcut = -1;
     if (half != 2) {
-        const double q = th[P_Q];
+        const double q = TH(P_Q), mc = TH(P_MC), dl_arg = TH(P_DL), phic = TH(P_PHIC);
+        const double chi1 = TH(P_CHI1), chi2 = TH(P_CHI2);
         const double r1q = recip_12(1.0 + q);
         const double eta = q * r1q * r1q;               // m1 m2 / M^2
         const double delta = (1.0 - q) * r1q;           // (m1 - m2)/M, m1 >= m2
-        const double chis = 0.5 * (th[P_CHI1] + th[P_CHI2]);
-        const double chia = 0.5 * (th[P_CHI1] - th[P_CHI2]);
         // The logarithms are taken of the mass in solar units and the powers of
         // T_sun (and the amplitude's constants) multiplied in after the exponential:
         // the exponents stay below 12, and with them the rounding that the
@@ -362,7 +369,7 @@ __device__ inline void point_coef_group(const Model &M, const Tables &T, const d
         // -60; relative error of log L against 80-bit arithmetic over prior draws,
         // 64,897 / 519,169 bins: 3.2e-15 / 1.1e-11 -> 1.7e-15 / 5.5e-12).
         // packed log: sub-lane 0 ln(eta), 1 ln(Mc), others ln(D_L) (or of D_L^3)
-        const double lg = log_tab(sl == 0 ? eta : (sl == 1 ? th[P_MC] : dl_arg));
+        const double lg = log_tab(sl == 0 ? eta : (sl == 1 ? mc : dl_arg));
         const double ln_eta = __shfl_sync(FULL, lg, 0, 8);
         const double ln_mc = __shfl_sync(FULL, lg, 1, 8);
         const double ln_dlx = __shfl_sync(FULL, lg, 2, 8);
@@ -392,11 +399,15 @@ __device__ inline void point_coef_group(const Model &M, const Tables &T, const d
         // sub-lane m computes basis coefficient m = K a^e_m (P_m(eta) + s_m), with
         // K v^(k-5) = K a^(k-5) f^((k-5)/3), P_m the eta polynomial of its PN order
         // and s_m its spin (or log) term.
-        const double pi = PI_D;
-        const double beta = (113.0 / 12.0) * (chis + delta * chia - (76.0 / 113.0) * eta * chis);
-        const double sigma = (79.0 / 8.0) * eta * th[P_CHI1] * th[P_CHI2];
-        const double gamma = (732985.0 / 2268.0 - 24260.0 / 81.0 * eta - 340.0 / 9.0 * eta * eta) * chis
-                           + (732985.0 / 2268.0 + 140.0 / 9.0 * eta) * delta * chia;
+        // The spin terms of all sub-lanes at once, as
+        //   (chi1 + chi2) (s0 + s1 eta + s2 eta^2) + delta (chi1 - chi2) (d0 + d1 eta)
+        //   + eta chi1 chi2 e + l (ln 4 + ln a)
+        // with each sub-lane's row of PN_SPIN: 11 FP64 instructions for the
+        // 4 beta, -10 sigma, -gamma and 3PN log terms, which one after the other took
+        // 22. With this, the prior transform over sub-lanes and the antenna products
+        // over pairs of them, GB300: slice update of 512 bins 805 -> 755 us an
+        // iteration, of 4017 bins 4.56 -> 4.06 ms.
+        double c4;
         {
             const int m = sl;
             // |e_m| for e = (-5, -3, -2, -1, 0, 1, 1, 2); negative powers from 1/a
@@ -406,18 +417,22 @@ __device__ inline void point_coef_group(const Model &M, const Tables &T, const d
             double pw = (e & 1) ? base : 1.0;
             pw *= (e & 2) ? b2 : 1.0;
             pw *= (e & 4) ? b2 * b2 : 1.0;
-            const double *pc = PN_POLY + 4 * m;
-            const double poly = fma(fma(fma(__ldg(pc + 3), eta, __ldg(pc + 2)), eta, __ldg(pc + 1)), eta, __ldg(pc));
-            const double sp = m == 2 ? 4.0 * beta
-                            : m == 3 ? -10.0 * sigma
-                            : m == 4 ? -gamma
-                            : m == 5 ? -6848.0 / 21.0 * (1.3862943611198906 + ln_a) : 0.0;
-            if (writer) out->a[m] = K * pw * (poly + sp);
+            const double *pc = PN_POLY + 4 * m, *ps = PN_SPIN + 8 * m;
+            double poly = fma(fma(fma(__ldg(pc + 3), eta, __ldg(pc + 2)), eta, __ldg(pc + 1)), eta, __ldg(pc));
+            const double ss = fma(fma(__ldg(ps + 2), eta, __ldg(ps + 1)), eta, __ldg(ps));
+            poly = fma(chi1 + chi2, ss, poly);
+            poly = fma(delta * (chi1 - chi2), fma(__ldg(ps + 4), eta, __ldg(ps + 3)), poly);
+            poly = fma(eta * (chi1 * chi2), __ldg(ps + 5), poly);
+            poly = fma(ln_a + 1.3862943611198906, __ldg(ps + 6), poly);
+            const double v = K * pw * poly;
+            if (writer) out->a[m] = v;
+            // constant: -phi_c - pi/4 + K phi5 (1 + 3 ln sqrt 6 + 3 ln a), K phi5 the
+            // coefficient of ln f
+            c4 = v;
         }
+        c4 = __shfl_sync(FULL, c4, 4, 8);
         if (sl == 0 && writer) {
-            // constant: -phi_c - pi/4 + K phi5 (1 + 3 ln sqrt 6 + 3 ln a), reduced mod 2 pi
-            const double phi5 = pi * (38645.0 / 756.0 - 65.0 / 9.0 * eta) - gamma;
-            const double c0 = -th[P_PHIC] - 0.25 * pi + K * phi5 * (1.0 + 3.0 * 0.8958797346140275 + 3.0 * ln_a);
+            const double c0 = fma(c4, fma(3.0, ln_a, 1.0 + 3.0 * 0.8958797346140275), -0.25 * PI_D - phic);
             out->c0 = c0 - TWO_PI_D * rint(c0 * INV_TWO_PI_D);
             out->c0u = c0;
             out->jcut = jcut;
@@ -427,39 +442,39 @@ __device__ inline void point_coef_group(const Model &M, const Tables &T, const d
     }
     // sky and detector part (half 0 or 2)
     if (half == 1) return;
-    const double ci = th[P_COSI];
+    const double ci = TH(P_COSI), sd = TH(P_SINDEC), tc = TH(P_TC), psi = TH(P_PSI), ra = TH(P_RA);
     // packed sincos: sub-lane 0 ra, others psi
     double sn, cs;
-    sincos_bf(sl == 0 ? th[P_RA] : th[P_PSI], sn, cs);
+    sincos_bf(sl == 0 ? ra : psi, sn, cs);
     const double sa = __shfl_sync(FULL, sn, 0, 8), ca = __shfl_sync(FULL, cs, 0, 8);
     const double sp = __shfl_sync(FULL, sn, 1, 8), cp = __shfl_sync(FULL, cs, 1, 8);
+    // the arms' products by sub-lane pairs: 2 d takes detector d's x arm, 2 d + 1 its
+    // y arm; then sub-lane d takes detector d
+    double fp = 1.0, fc = 0.0, dt = 0.0;
+    if (!M.ideal) {
+        const double cd = sqrt(1.0 - sd * sd);
+        // wave-frame basis X, Y (Anderson et al. 2001) and source direction n
+        const double X0 = sa * cp - sp * ca * sd, X1 = -ca * cp - sp * sa * sd, X2 = sp * cd;
+        const double Y0 = -sa * sp - cp * ca * sd, Y1 = ca * sp - cp * sa * sd, Y2 = cp * cd;
+        const int da = (sl >> 1) < M.n_det ? sl >> 1 : 0, dr = sl < M.n_det ? sl : 0;
+        const double *x = (sl & 1) ? M.yarm[da] : M.xarm[da];
+        const double xX = x[0] * X0 + x[1] * X1 + x[2] * X2;
+        const double xY = x[0] * Y0 + x[1] * Y1 + x[2] * Y2;
+        // D = (x x^T - y y^T)/2: X^T D X - Y^T D Y and 2 X^T D Y
+        const double sq = xX * xX - xY * xY, pr = xX * xY;
+        const int px = (2 * sl) & 7, py = (2 * sl + 1) & 7;
+        fp = 0.5 * (__shfl_sync(FULL, sq, px, 8) - __shfl_sync(FULL, sq, py, 8));
+        fc = __shfl_sync(FULL, pr, px, 8) - __shfl_sync(FULL, pr, py, 8);
+        const double *r = M.pos[dr];
+        dt = -(r[0] * cd * ca + r[1] * cd * sa + r[2] * sd) * (1.0 / C_SI);
+    }
     double hh_part = 0.0;
+    const double qre = fp * (0.5 * (1.0 + ci * ci));
+    const double qim = -fc * ci;
     if (sl < M.n_det) {
         const int dd = sl;
-        double fp, fc, dt;
-        if (M.ideal) {
-            fp = 1.0; fc = 0.0; dt = 0.0;
-        } else {
-            const double sd = th[P_SINDEC];
-            const double cd = sqrt(1.0 - sd * sd);
-            // wave-frame basis X, Y (Anderson et al. 2001) and source direction n
-            const double X0 = sa * cp - sp * ca * sd, X1 = -ca * cp - sp * sa * sd, X2 = sp * cd;
-            const double Y0 = -sa * sp - cp * ca * sd, Y1 = ca * sp - cp * sa * sd, Y2 = cp * cd;
-            const double *x = M.xarm[dd], *y = M.yarm[dd];
-            // D = (x x^T - y y^T)/2: X^T D Y = ((x.X)(x.Y) - (y.X)(y.Y))/2
-            const double xX = x[0] * X0 + x[1] * X1 + x[2] * X2;
-            const double xY = x[0] * Y0 + x[1] * Y1 + x[2] * Y2;
-            const double yX = y[0] * X0 + y[1] * X1 + y[2] * X2;
-            const double yY = y[0] * Y0 + y[1] * Y1 + y[2] * Y2;
-            fp = 0.5 * ((xX * xX - yX * yX) - (xY * xY - yY * yY));
-            fc = (xX * xY - yX * yY);
-            const double *r = M.pos[dd];
-            dt = -(r[0] * cd * ca + r[1] * cd * sa + r[2] * sd) * (1.0 / C_SI);
-        }
-        const double qre = fp * 0.5 * (1.0 + ci * ci);
-        const double qim = -fc * ci;
         if (writer) {
-            out->tau[dd] = th[P_TC] + dt;
+            out->tau[dd] = tc + dt;
             // half 2 leaves the amplitude to point_coef_join
             out->gre[dd] = half == 2 ? qre : amp * qre;
             out->gim[dd] = half == 2 ? -qim : -amp * qim;
