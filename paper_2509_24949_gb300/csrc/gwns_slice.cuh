@@ -397,18 +397,55 @@ enum { PH_NEWSTEP = 0, PH_OUT = 1, PH_SHRINK = 2, PH_DONE = 3, PH_WALK = 4 };
 enum { KIND_L = 0, KIND_R = 1, KIND_SH = 2, KIND_W = 3 };
 constexpr int CACHE_MAX = 16;
 
+// Planned candidates and evaluated, not yet consumed ones, in shared memory: a
+// plan writes its entries behind the n kept ones, the coefficient stage reads the
+// points there, and the results join them. One copy per lane in local memory, 900
+// bytes a thread, took up to 110 KB of each SM's L1 and its latency at every
+// transition; with it here, found by one ballot, and the positions and points kept
+// instead of computed again when a result is consumed (24 FP64 instructions a
+// candidate), GB300: slice update of 512 bins FP64 755 -> 674 us, 4017 bins FP64
+// 4.06 -> 3.70 ms, 64,897 bins mixed 10.9 -> 10.4 ms; four served analyses 286 -> 241 ms.
+struct CandCache {
+    double y[CACHE_MAX][MAXD];     // the point
+    double val[CACHE_MAX];         // log L
+    double t[CACHE_MAX];           // slice sampling: the position on the line
+    int key[CACHE_MAX];            // kind << 16 | index
+    int bins[CACHE_MAX];
+};
+
+__device__ __forceinline__ int cand_key(int kind, int idx) { return (kind << 16) | idx; }
+
 struct Chain {
-    double x, e, lrow[MAXD];
+    double x, e;
     double lx, a, b;
     int s, phase, nl, nr, nsh, caps, left_done, right_done;
     long long evals;
     unsigned long long bins, bins_lo;   // bins read by the consumed evaluations; of those, in low-degree groups
-    // cache of evaluated, not yet consumed candidates
     int ncache;
-    int ckind[CACHE_MAX], cidx[CACHE_MAX], cbins[CACHE_MAX];
-    double cval[CACHE_MAX];
-    double cy[CACHE_MAX];      // random walk: the evaluated proposal (lane's coordinate)
+    // the candidate that chain_run stopped at, for the plan
+    double next_t, next_y;
 };
+
+// A chain between its rounds, in shared memory, so that its state takes no
+// registers of the bin sums.
+struct ChainStore {
+    double x[MAXD], e[MAXD];
+    Chain c;        // with x and e of lane 0
+};
+__device__ __forceinline__ void chain_load(const ChainStore &q, Chain &c, int lane, int d) {
+    c = q.c;
+    c.x = lane < d ? q.x[lane] : 0.0;
+    c.e = lane < d ? q.e[lane] : 0.0;
+}
+__device__ __forceinline__ void chain_save(ChainStore &q, const Chain &c, int lane, int d) {
+    __syncwarp();
+    if (lane < d) {
+        q.x[lane] = c.x;
+        q.e[lane] = c.e;
+    }
+    if (lane == 0) q.c = c;
+    __syncwarp();
+}
 
 // A consumed evaluation's bins (jcut + 1 of them): all, and those at or past lo_bin.
 __device__ __forceinline__ void count_bins(Chain &c, int bins, long long lo_bin) {
@@ -426,34 +463,46 @@ __device__ __forceinline__ double line_y(const Model &M, const Chain &c, double 
 }
 
 __device__ __forceinline__ bool warp_inbox(double y, int lane, int d) {
-    return __all_sync(0xffffffffu, lane >= d || (y >= 0.0 && y <= 1.0));
+    // 0 <= y <= 1 by the bits (and -0): an FP64 comparison costs 64 cycles
+    const unsigned long long b = (unsigned long long)__double_as_longlong(y);
+    return __all_sync(0xffffffffu, lane >= d || b <= 0x3ff0000000000000ull || b == 0x8000000000000000ull);
 }
 
-__device__ __forceinline__ int cache_find(const Chain &c, int kind, int idx) {
-    for (int i = 0; i < c.ncache; i++)
-        if (c.ckind[i] == kind && c.cidx[i] == idx) return i;
-    return -1;
+// Index of an entry (all lanes), -1 if absent: one key per lane.
+__device__ __forceinline__ int cache_find(const Chain &c, const CandCache &q, int kind, int idx) {
+    const int lane = threadIdx.x & 31;
+    const unsigned m = __ballot_sync(0xffffffffu, lane < c.ncache && q.key[lane & (CACHE_MAX - 1)] == cand_key(kind, idx));
+    return (int)__ffs(m) - 1;
 }
 
-__device__ __forceinline__ void cache_drop(Chain &c, int i) {
-    c.ncache--;
-    c.ckind[i] = c.ckind[c.ncache];
-    c.cidx[i] = c.cidx[c.ncache];
-    c.cval[i] = c.cval[c.ncache];
-    c.cbins[i] = c.cbins[c.ncache];
-    c.cy[i] = c.cy[c.ncache];
+// Drop entry i: the last one takes its place.
+__device__ __forceinline__ void cache_drop(Chain &c, CandCache &q, int i) {
+    const int lane = threadIdx.x & 31;
+    const int l = --c.ncache;
+    __syncwarp();
+    if (i != l) {
+        if (lane < MAXD) q.y[i][lane] = q.y[l][lane];
+        if (lane == 0) {
+            q.val[i] = q.val[l];
+            q.t[i] = q.t[l];
+            q.key[i] = q.key[l];
+            q.bins[i] = q.bins[l];
+        }
+    }
+    __syncwarp();
 }
 
-// Drop every cached result of one stepping-out side (once that side has ended,
-// its later candidates are never consumed).
-__device__ __forceinline__ void cache_purge(Chain &c, int kind) {
+// Drop every cached result of one kind (once a stepping-out side has ended, its
+// later candidates are never consumed).
+__device__ __forceinline__ void cache_purge(Chain &c, CandCache &q, int kind) {
     for (int i = c.ncache - 1; i >= 0; i--)
-        if (c.ckind[i] == kind) cache_drop(c, i);
+        if ((q.key[i] >> 16) == kind) cache_drop(c, q, i);
 }
 
-__device__ __forceinline__ void end_side(Chain &c, bool left) {
-    if (left) { c.left_done = 1; cache_purge(c, KIND_L); }
-    else { c.right_done = 1; cache_purge(c, KIND_R); }
+__device__ __forceinline__ void end_side(Chain &c, CandCache &q, bool left) {
+    if (left) c.left_done = 1;
+    else c.right_done = 1;
+    cache_purge(c, q, left ? KIND_L : KIND_R);
 }
 
 __device__ __forceinline__ double shrink_t(const StepArgs &A, double a, double b, int nsh, int step,
@@ -463,10 +512,8 @@ __device__ __forceinline__ double shrink_t(const StepArgs &A, double a, double b
 }
 
 // Hit-and-run direction of slice step s: lane i < d gets coordinate i of
-// L z / |z|, z ~ N(0, I) by Box-Muller (two normals per draw); lrow is the
-// lane's row of the Cholesky factor L.
-__device__ __forceinline__ double slice_direction(const StepArgs &A, const double *lrow, int chain, uint32_t iter,
-                                                  int s, int lane, int d) {
+// L z / |z|, z ~ N(0, I) by Box-Muller (two normals per draw), L the Cholesky factor.
+static __device__ __noinline__ double slice_direction(const StepArgs &A, int chain, uint32_t iter, int s, int lane, int d) {
     double z = 0.0;
     if (lane < d) {
         const uint4 w = draw(A.seed, (uint32_t)(lane >> 1), (uint32_t)s, (uint32_t)chain, iter);
@@ -480,7 +527,7 @@ __device__ __forceinline__ double slice_direction(const StepArgs &A, const doubl
     double acc = 0.0;
     for (int j = 0; j < d; j++) {
         const double zj = __shfl_sync(0xffffffffu, z, j);
-        if (j <= lane) acc = __dadd_rn(acc, __dmul_rn(lrow[j], zj));
+        if (j <= lane && lane < d) acc = __dadd_rn(acc, __dmul_rn(A.chol[lane * d + j], zj));
     }
     return (lane < d) ? acc / nz : 0.0;
 }
@@ -489,7 +536,7 @@ __device__ __forceinline__ double slice_direction(const StepArgs &A, const doubl
 // bracket draws), cap and prior-box outcomes, and results already in the cache.
 // Returns when the next transition needs an evaluation not in the cache, or the
 // chain is done.
-static __device__ void chain_run(const Model &M, const StepArgs &A, Chain &c, int chain, uint32_t iter,
+static __device__ void chain_run(const Model &M, const StepArgs &A, Chain &c, CandCache &q, int chain, uint32_t iter,
                                  double lstar, const double *e_pre, int e_pre_step) {
     const int lane = threadIdx.x & 31, d = M.dim;
     for (int guard = 0; guard < (1 << 22); guard++) {
@@ -498,7 +545,7 @@ static __device__ void chain_run(const Model &M, const StepArgs &A, Chain &c, in
             if (c.s >= A.steps) { c.phase = PH_DONE; return; }
             // direction (computed ahead by a spare warp when it could be)
             if (e_pre_step == c.s) c.e = (lane < d) ? e_pre[lane] : 0.0;
-            else c.e = slice_direction(A, c.lrow, chain, iter, c.s, lane, d);
+            else c.e = slice_direction(A, chain, iter, c.s, lane, d);
             const uint4 w = draw(A.seed, SLOT_OFFSET, (uint32_t)c.s, (uint32_t)chain, iter);
             const double r = u01(w.x, w.y);
             c.a = -r;
@@ -514,23 +561,23 @@ static __device__ void chain_run(const Model &M, const StepArgs &A, Chain &c, in
             if (!left && c.right_done) { c.phase = PH_SHRINK; continue; }
             const int n = left ? c.nl : c.nr;
             if (n >= A.max_stepout) {
-                end_side(c, left);
+                end_side(c, q, left);
                 continue;
             }
-            const double t = left ? c.a : c.b;
-            const double y = line_y(M, c, t, lane, d);
-            if (!warp_inbox(y, lane, d)) {
-                end_side(c, left);
+            const int ci = cache_find(c, q, left ? KIND_L : KIND_R, n);
+            if (ci < 0) {
+                c.next_t = left ? c.a : c.b;
+                c.next_y = line_y(M, c, c.next_t, lane, d);
+                if (warp_inbox(c.next_y, lane, d)) return;
+                end_side(c, q, left);
                 continue;
             }
-            const int ci = cache_find(c, left ? KIND_L : KIND_R, n);
-            if (ci < 0) return;
-            const bool in = c.cval[ci] > lstar;
+            const bool in = q.val[ci] > lstar;
             c.evals++;
-            count_bins(c, c.cbins[ci], A.lo_bin);
-            cache_drop(c, ci);
-            if (left) { if (in) { c.a -= 1.0; c.nl++; } else end_side(c, true); }
-            else { if (in) { c.b += 1.0; c.nr++; } else end_side(c, false); }
+            count_bins(c, q.bins[ci], A.lo_bin);
+            cache_drop(c, q, ci);
+            if (left) { if (in) { c.a -= 1.0; c.nl++; } else end_side(c, q, true); }
+            else { if (in) { c.b += 1.0; c.nr++; } else end_side(c, q, false); }
             continue;
         }
         // PH_SHRINK
@@ -540,15 +587,24 @@ static __device__ void chain_run(const Model &M, const StepArgs &A, Chain &c, in
             c.phase = PH_NEWSTEP;
             continue;
         }
-        const double t = shrink_t(A, c.a, c.b, c.nsh, c.s, chain, iter);
-        const double y = line_y(M, c, t, lane, d);
-        if (warp_inbox(y, lane, d)) {
-            const int ci = cache_find(c, KIND_SH, c.nsh);
-            if (ci < 0) return;
-            const double val = c.cval[ci];
+        // an evaluated candidate comes with its position and point: planned as the
+        // next draw after rejections, which is how it is reached
+        const int ci = cache_find(c, q, KIND_SH, c.nsh);
+        double t;
+        if (ci < 0) {
+            t = shrink_t(A, c.a, c.b, c.nsh, c.s, chain, iter);
+            const double y = line_y(M, c, t, lane, d);
+            if (warp_inbox(y, lane, d)) {
+                c.next_t = t;
+                c.next_y = y;
+                return;
+            }
+        } else {
+            t = q.t[ci];
+            const double val = q.val[ci], y = (lane < d) ? q.y[ci][lane] : 0.5;
             c.evals++;
-            count_bins(c, c.cbins[ci], A.lo_bin);
-            cache_drop(c, ci);
+            count_bins(c, q.bins[ci], A.lo_bin);
+            cache_drop(c, q, ci);
             if (val > lstar) {
                 c.x = y;
                 c.lx = val;
@@ -563,12 +619,21 @@ static __device__ void chain_run(const Model &M, const StepArgs &A, Chain &c, in
     c.phase = PH_DONE;   // unreachable with finite caps; keeps the loop bounded
 }
 
+// Candidate ns of a plan: its point, position and key behind the cache's entries.
+__device__ __forceinline__ void plan_put(const Chain &c, CandCache &q, int ns, int key, double t, double y, int lane, int d) {
+    const int i = c.ncache + ns;
+    if (lane < d) q.y[i][lane] = y;
+    if (lane == 0) {
+        q.t[i] = t;
+        q.key[i] = key;
+    }
+}
+
 // Plan up to S candidates to evaluate in the next round (in-box, not cached),
-// continuing the current stage's sequences. Writes their coordinates to
-// ysh[slot][*] and their keys to pk/pi; returns the number of slots used.
+// continuing the current stage's sequences; returns their number.
 template <int S>
-__device__ int chain_plan(const Model &M, const StepArgs &A, const Chain &c, int chain, uint32_t iter,
-                          double (*ysh)[MAXD], int *pk, int *pidx, int depth) {
+__device__ int chain_plan(const Model &M, const StepArgs &A, const Chain &c, CandCache &q, int chain, uint32_t iter,
+                          int depth) {
     const int lane = threadIdx.x & 31, d = M.dim;
     int ns = 0;
     const int room = CACHE_MAX - c.ncache;
@@ -582,16 +647,16 @@ __device__ int chain_plan(const Model &M, const StepArgs &A, const Chain &c, int
             const bool left = (side == 0);
             if (left ? c.left_done : c.right_done) continue;
             const int limit = (left && !c.right_done) ? (cap + 1) / 2 : cap;
+            const int kind = left ? KIND_L : KIND_R;
             double t = left ? c.a : c.b;
             const int n0 = left ? c.nl : c.nr;
             for (int n = n0; n < n0 + S && n < A.max_stepout && ns < limit; n++) {
-                const double y = line_y(M, c, t, lane, d);
-                if (!warp_inbox(y, lane, d)) break;
-                if (cache_find(c, left ? KIND_L : KIND_R, n) < 0) {
-                    if (lane < d) ysh[ns][lane] = y;
-                    pk[ns] = left ? KIND_L : KIND_R;
-                    pidx[ns] = n;
-                    ns++;
+                if (cache_find(c, q, kind, n) < 0) {
+                    // the side in progress stopped at its first candidate
+                    const bool next = n == n0 && (left || c.left_done);
+                    const double y = next ? c.next_y : line_y(M, c, t, lane, d);
+                    if (!next && !warp_inbox(y, lane, d)) break;
+                    plan_put(c, q, ns++, cand_key(kind, n), t, y, lane, d);
                 }
                 if (left) t -= 1.0; else t += 1.0;
             }
@@ -599,13 +664,15 @@ __device__ int chain_plan(const Model &M, const StepArgs &A, const Chain &c, int
     } else if (c.phase == PH_SHRINK) {
         double a = c.a, b = c.b;
         for (int n = c.nsh; n < c.nsh + S && n < A.max_shrink && ns < cap; n++) {
-            const double t = shrink_t(A, a, b, n, c.s, chain, iter);
-            const double y = line_y(M, c, t, lane, d);
-            if (warp_inbox(y, lane, d) && cache_find(c, KIND_SH, n) < 0) {
-                if (lane < d) ysh[ns][lane] = y;
-                pk[ns] = KIND_SH;
-                pidx[ns] = n;
-                ns++;
+            double t;
+            const int ci = n == c.nsh ? -1 : cache_find(c, q, KIND_SH, n);
+            if (ci >= 0) {
+                t = q.t[ci];
+            } else {
+                const bool next = n == c.nsh;
+                t = next ? c.next_t : shrink_t(A, a, b, n, c.s, chain, iter);
+                const double y = next ? c.next_y : line_y(M, c, t, lane, d);
+                if (next || warp_inbox(y, lane, d)) plan_put(c, q, ns++, cand_key(KIND_SH, n), t, y, lane, d);
             }
             if (t < 0.0) a = t; else b = t;     // as if rejected
         }
@@ -622,8 +689,7 @@ __device__ int chain_plan(const Model &M, const StepArgs &A, const Chain &c, int
 // between iterations (k_finish). Speculation: the proposals after the current
 // one are evaluated from the current point, as if it were rejected; an
 // acceptance discards them. c.s counts accepted moves, c.nsh the proposal.
-__device__ __forceinline__ double walk_disp(const StepArgs &A, const Chain &c, int chain, uint32_t iter, int p,
-                                            int lane, int d) {
+static __device__ __noinline__ double walk_disp(const StepArgs &A, int chain, uint32_t iter, int p, int lane, int d) {
     double z = 0.0;
     if (lane < d) {
         const uint4 w = draw(A.seed, (uint32_t)(lane >> 1), (uint32_t)p, (uint32_t)chain, iter);
@@ -636,7 +702,7 @@ __device__ __forceinline__ double walk_disp(const StepArgs &A, const Chain &c, i
     double acc = 0.0;
     for (int j = 0; j < d; j++) {
         const double zj = __shfl_sync(0xffffffffu, z, j);
-        if (j <= lane) acc = __dadd_rn(acc, __dmul_rn(c.lrow[j], zj));
+        if (j <= lane && lane < d) acc = __dadd_rn(acc, __dmul_rn(A.chol[lane * d + j], zj));
     }
     return __dmul_rn(acc, A.walk_scale);
 }
@@ -648,7 +714,7 @@ __device__ __forceinline__ double walk_y(const Model &M, const Chain &c, double 
     return y;
 }
 
-static __device__ void walk_run(const Model &M, const StepArgs &A, Chain &c, int chain, uint32_t iter,
+static __device__ void walk_run(const Model &M, const StepArgs &A, Chain &c, CandCache &q, int chain, uint32_t iter,
                                 double lstar, int walk_len) {
     const int lane = threadIdx.x & 31, d = M.dim;
     for (int guard = 0; guard < (1 << 22); guard++) {
@@ -657,24 +723,24 @@ static __device__ void walk_run(const Model &M, const StepArgs &A, Chain &c, int
         // an evaluated proposal comes with its point (planned from the current
         // point: the cache is emptied at every acceptance); otherwise compute
         // it, skip it outside the box, or wait for its evaluation
-        const int ci = cache_find(c, KIND_W, c.nsh);
+        const int ci = cache_find(c, q, KIND_W, c.nsh);
         double y;
         if (ci >= 0) {
-            y = (lane < d) ? c.cy[ci] : 0.5;
+            y = (lane < d) ? q.y[ci][lane] : 0.5;
         } else {
-            y = walk_y(M, c, walk_disp(A, c, chain, iter, c.nsh, lane, d), lane, d);
+            y = walk_y(M, c, walk_disp(A, chain, iter, c.nsh, lane, d), lane, d);
             if (!warp_inbox(y, lane, d)) { c.nsh++; continue; }
             return;
         }
-        const double val = c.cval[ci];
+        const double val = q.val[ci];
         c.evals++;
-        count_bins(c, c.cbins[ci], A.lo_bin);
-        cache_drop(c, ci);
+        count_bins(c, q.bins[ci], A.lo_bin);
+        cache_drop(c, q, ci);
         if (val > lstar) {
             c.x = y;
             c.lx = val;
             c.s++;
-            cache_purge(c, KIND_W);
+            cache_purge(c, q, KIND_W);
         }
         c.nsh++;
     }
@@ -682,22 +748,17 @@ static __device__ void walk_run(const Model &M, const StepArgs &A, Chain &c, int
 }
 
 template <int S>
-__device__ int walk_plan(const Model &M, const StepArgs &A, const Chain &c, int chain, uint32_t iter,
-                         double (*ysh)[MAXD], int *pk, int *pidx, int depth, int walk_len) {
+__device__ int walk_plan(const Model &M, const StepArgs &A, const Chain &c, CandCache &q, int chain, uint32_t iter,
+                         int depth, int walk_len) {
     const int lane = threadIdx.x & 31, d = M.dim;
     const int room = CACHE_MAX - c.ncache;
     const int lim = depth < S ? depth : S;
     const int cap = lim < room ? lim : room;
     int ns = 0;
     for (int p = c.nsh; p < c.nsh + S && p < walk_len && ns < cap; p++) {
-        if (cache_find(c, KIND_W, p) >= 0) continue;
-        const double y = walk_y(M, c, walk_disp(A, c, chain, iter, p, lane, d), lane, d);
-        if (warp_inbox(y, lane, d)) {
-            if (lane < d) ysh[ns][lane] = y;
-            pk[ns] = KIND_W;
-            pidx[ns] = p;
-            ns++;
-        }
+        if (cache_find(c, q, KIND_W, p) >= 0) continue;
+        const double y = walk_y(M, c, walk_disp(A, chain, iter, p, lane, d), lane, d);
+        if (warp_inbox(y, lane, d)) plan_put(c, q, ns++, cand_key(KIND_W, p), 0.0, y, lane, d);
     }
     return ns;
 }
@@ -926,9 +987,10 @@ template <int PREC, int NDET, int S, int W = S, int FORM = FORM_BOTH, bool WS = 
 __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, const int chain) {
     __shared__ Coef coef[S];
     __shared__ CoefMixed cm[S];
-    __shared__ double ysh[S][MAXD];
+    __shared__ CandCache cq;
+    __shared__ ChainStore cs;
     __shared__ double lval[S];
-    __shared__ int nslot, tailmode;
+    __shared__ int nslot, nbase, tailmode;
     __shared__ double e_next[MAXD];         // direction of slice step e_next_step, computed ahead
     __shared__ int e_next_step, cur_step;
     __shared__ int jc[S];
@@ -943,9 +1005,8 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
     const uint32_t iter = (uint32_t)A.state->iter;
     const double lstar = A.state->lstar;
     const int walk_len = A.state->walk_len;
-    Chain c;
-    int pk[S], pidx[S];
     if (warp == 0) {
+        Chain c;
         const int m = A.n - A.k;
         const uint4 w = draw(A.seed, 0u, STEP_START, (uint32_t)chain, iter);
         int idx = (int)(u01(w.x, w.y) * m);
@@ -953,20 +1014,24 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
         const int src = A.order[A.k + idx];
         c.x = (lane < d) ? A.live_u[(size_t)src * d + lane] : 0.0;
         c.lx = A.live_logl[src];
-        for (int j = 0; j < MAXD; j++) c.lrow[j] = (lane < d && j < d) ? A.chol[lane * d + j] : 0.0;
         c.e = 0.0; c.a = 0.0; c.b = 0.0;
         c.s = 0; c.phase = A.kernel == 1 ? PH_WALK : PH_NEWSTEP; c.nl = c.nr = c.nsh = 0; c.caps = 0;
         c.evals = 0; c.bins = 0; c.bins_lo = 0;
         c.left_done = c.right_done = 0; c.ncache = 0;
+        c.next_t = c.next_y = 0.0;
+        chain_save(cs, c, lane, d);
         if (lane == 0) e_next_step = -1;
+        __syncwarp();
     }
     for (;;) {
         if (warp == 0) {
+            Chain c;
+            chain_load(cs, c, lane, d);
             // a bounded wait of the work-shared update gave up (status bit 1):
             // every chain ends at its current point, so that the launch ends
             if (WS && (*((volatile int *)&A.state->status) & 2)) c.phase = PH_DONE;
-            if (A.kernel == 1) walk_run(M, A, c, chain, iter, lstar, walk_len);
-            else chain_run(M, A, c, chain, iter, lstar, e_next, e_next_step);
+            if (A.kernel == 1) walk_run(M, A, c, cq, chain, iter, lstar, walk_len);
+            else chain_run(M, A, c, cq, chain, iter, lstar, e_next, e_next_step);
             // plan the base depth while many chains run; the stragglers of the
             // update (fewer running chains than the tail threshold) use every warp.
             // FP64 on fine grids splits every candidate's bins over two warps in
@@ -981,19 +1046,21 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                 tail = 2;
             }
             int ns = (c.phase == PH_DONE) ? 0
-                   : A.kernel == 1 ? walk_plan<S>(M, A, c, chain, iter, ysh, pk, pidx, depth, walk_len)
-                                   : chain_plan<S>(M, A, c, chain, iter, ysh, pk, pidx, depth);
+                   : A.kernel == 1 ? walk_plan<S>(M, A, c, cq, chain, iter, depth, walk_len)
+                                   : chain_plan<S>(M, A, c, cq, chain, iter, depth);
             if (ns == 0 && c.phase != PH_DONE) {
                 // cannot happen with the bounds above; end the chain at its
                 // current (in-slice) point and flag the run state
                 c.phase = PH_DONE;
                 if (lane == 0) atomicOr(&A.state->status, 1);
             }
-            if (lane == 0) { nslot = ns; tailmode = tail; cur_step = c.s; }
+            if (lane == 0) { nslot = ns; nbase = c.ncache; tailmode = tail; cur_step = c.s; }
+            chain_save(cs, c, lane, d);
         }
         __syncthreads();
         const int ns = nslot;
         if (ns == 0) break;
+        const double (*ysh)[MAXD] = cq.y + nbase;       // the round's points
         // coefficients: candidates 4j .. 4j+3 (8 lanes each) by one warp, or,
         // with two warps per group of four, the mass/phase half on warp 2j and
         // the sky/detector half on warp 2j + 1 (independent FP64 chains on two
@@ -1014,9 +1081,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                 // a warp without coefficients computes the next slice step's direction
                 const int s1 = cur_step + 1;
                 if (s1 < A.steps && e_next_step != s1) {
-                    double lrow[MAXD];
-                    for (int j = 0; j < MAXD; j++) lrow[j] = (lane < d && j < d) ? A.chol[lane * d + j] : 0.0;
-                    const double e1 = slice_direction(A, lrow, chain, iter, s1, lane, d);
+                    const double e1 = slice_direction(A, chain, iter, s1, lane, d);
                     if (lane < d) e_next[lane] = e1;
                     __syncwarp();
                     if (lane == 0) e_next_step = s1;
@@ -1182,18 +1247,18 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
         }
         __syncthreads();
         if (warp == 0) {
-            for (int sl = 0; sl < ns; sl++) {
-                c.ckind[c.ncache] = pk[sl];
-                c.cidx[c.ncache] = pidx[sl];
-                c.cval[c.ncache] = lval[sl];
-                c.cbins[c.ncache] = coef[sl].jcut + 1;
-                c.cy[c.ncache] = (lane < d) ? ysh[sl][lane] : 0.5;
-                c.ncache++;
+            if (lane < ns) {
+                cq.val[nbase + lane] = lval[lane];
+                cq.bins[nbase + lane] = coef[lane].jcut + 1;
             }
+            if (lane == 0) cs.c.ncache = nbase + ns;
+            __syncwarp();
         }
         // coef/lval are rewritten only after the next barrier's plan
     }
     if (warp == 0) {
+        Chain c;
+        chain_load(cs, c, lane, d);
         const int dst = A.order[chain];
         if (lane < d) A.live_u[(size_t)dst * d + lane] = c.x;
         if (lane == 0) {
