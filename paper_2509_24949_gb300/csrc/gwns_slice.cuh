@@ -955,35 +955,19 @@ __device__ void ws_help(const Model &M, const Tables &T, const StepArgs &A) {
     }
 }
 
-// Forms of the tiled mixed sums a kernel compiles. FORM_BOTH chooses at run
-// time: rotation (tile_bins_rot) on tiles of 32 bins or more, direct on
-// shorter ones. FORM_DIRECT and FORM_ROT compile one form only (the serving
-// kernel, which runs many analyses per launch, spilled registers with both);
-// FORM_ROT kernels run only grids with tiles of 32 bins or more.
-enum { FORM_DIRECT = 0, FORM_BOTH = 1, FORM_ROT = 2 };
-
-template <int FORM>
-__device__ __forceinline__ bool form_rot(const Model &M) {
-    if constexpr (FORM == FORM_ROT) return true;
-    else if constexpr (FORM == FORM_DIRECT) return false;
-    else return M.tlg >= 5;
-}
+// Form of the tiled mixed sums a kernel compiles: FORM_ROT, rotation
+// (tile_bins_rot), for grids with tiles of 32 bins or more only; FORM_DIRECT for
+// all others (shorter tiles, per-bin grids, FP64).
+enum { FORM_DIRECT = 0, FORM_ROT = 2 };
 
 template <int NDET, int NC, int FORM>
 __device__ __forceinline__ void tile_bins_form(const Model &M, const Tables &T, const CoefMixed *cm,
                                                const int *jc, int nc, int g0, int gstride,
                                                float zh[NC][NDET][2], float zl[NC][NDET][2]) {
-    if constexpr (FORM == FORM_ROT) {
-        tile_bins<NDET, NC, true>(T, M.tlg, M.np, cm, jc, nc, g0, gstride, zh, zl);
-    } else if constexpr (FORM == FORM_DIRECT) {
-        tile_bins<NDET, NC, false>(T, M.tlg, M.np, cm, jc, nc, g0, gstride, zh, zl);
-    } else {
-        if (M.tlg >= 5) tile_bins<NDET, NC, true>(T, M.tlg, M.np, cm, jc, nc, g0, gstride, zh, zl);
-        else tile_bins<NDET, NC, false>(T, M.tlg, M.np, cm, jc, nc, g0, gstride, zh, zl);
-    }
+    tile_bins<NDET, NC, FORM == FORM_ROT>(T, M.tlg, M.np, cm, jc, nc, g0, gstride, zh, zl);
 }
 
-template <int PREC, int NDET, int S, int W = S, int FORM = FORM_BOTH, bool WS = false>
+template <int PREC, int NDET, int S, int W, int FORM, bool WS = false>
 __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, const int chain) {
     __shared__ Coef coef[S];
     __shared__ CoefMixed cm[S];
@@ -1074,7 +1058,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                 const int cnt = ns - 4 * grp < 4 ? ns - 4 * grp : 4;
                 if (PREC == 1 && M.cdf)
                     point_coef_group_mx(M, T, ysh[4 * grp], MAXD, &coef[4 * grp], &cm[4 * grp], cnt,
-                                        form_rot<FORM>(M), 1 + (warp & 1));
+                                        FORM == FORM_ROT, 1 + (warp & 1));
                 else
                     point_coef_group(M, T, ysh[4 * grp], MAXD, &coef[4 * grp], cnt, 1 + (warp & 1));
             } else if (warp == W - 1 && A.kernel == 0) {
@@ -1098,7 +1082,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                 const int cnt = ns - 4 * warp < 4 ? ns - 4 * warp : 4;
                 if (PREC == 1 && M.cdf)
                     point_coef_group_mx(M, T, ysh[4 * warp], MAXD, &coef[4 * warp], &cm[4 * warp], cnt,
-                                        form_rot<FORM>(M));
+                                        FORM == FORM_ROT);
                 else
                     point_coef_group(M, T, ysh[4 * warp], MAXD, &coef[4 * warp], cnt);
                 if (use_fx) {
@@ -1126,14 +1110,14 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             // mixed, every warp on every candidate of the round: the tiled form
             // shares out the tile groups (two candidates per pass on one table
             // load), the per-bin form strides the bins
-            if (warp < ns && !M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, form_rot<FORM>(M));
+            if (warp < ns && !M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, FORM == FORM_ROT);
             if (lane == 0 && warp < ns) jc[warp] = coef[warp].jcut;
             __syncthreads();
             if (WS) {
                 // work-shared: fixed chunks of tile groups, computed by this CTA's
                 // warps and by helper CTAs, summed in chunk order into part[0]
                 ws_owner_round<NDET, W>(M, T, A, cm, jc, ns, part[0]);
-            } else if (M.tlg) {
+            } else if (FORM == FORM_ROT || M.tlg) {
                 // the (candidate pair, tile group) items of the round are dealt out
                 // to the warps in turn, pair after pair, so that every warp has
                 // work when a candidate spans fewer groups than there are warps
@@ -1229,15 +1213,15 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                     bins_fx<NDET>(T, fx[warp], sct, lane, 32, zh, zl);
                     v = warp_detector_terms_df<NDET>(zh, zl, coef[warp], T.fxs);
                 }
-            } else if (M.tlg) {
-                if (!M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, form_rot<FORM>(M));
+            } else if (FORM == FORM_ROT || M.tlg) {
+                if (!M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, FORM == FORM_ROT);
                 if (lane == 0) jc[warp] = coef[warp].jcut;
                 __syncwarp();
                 float zh[1][NDET][2], zl[1][NDET][2];
                 tile_bins_form<NDET, 1, FORM>(M, T, &cm[warp], &jc[warp], 1, 0, 1, zh, zl);
                 v = warp_detector_terms_df<NDET>(zh[0], zl[0], coef[warp]);
             } else {
-                if (!M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, form_rot<FORM>(M));
+                if (!M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, FORM == FORM_ROT);
                 __syncwarp();
                 float zh[NDET][2], zl[NDET][2];
                 bins_mixed<NDET>(T, M.N, cm[warp], coef[warp].jcut, lane, 32, zh, zl);
@@ -1279,9 +1263,23 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
 // spite of ~100 bytes of spills in the mixed tile loop.
 #define SLICE_MIN_BLOCKS(PREC, S) (16 / (S))
 
-template <int PREC, int NDET, int S, int W = S>
+template <int PREC, int NDET, int S, int W, int FORM>
 __global__ void __launch_bounds__(W * 32, SLICE_MIN_BLOCKS(PREC, W)) k_slice(Model M, Tables T, StepArgs A) {
-    slice_body<PREC, NDET, S, W>(M, T, A, blockIdx.x);
+    slice_body<PREC, NDET, S, W, FORM>(M, T, A, blockIdx.x);
+}
+
+// One form of the tiled mixed sums per kernel, as in the serving kernels: with
+// both, a chain's hot code is longer and its registers spill (GB300, 64,897 bins,
+// slice update of 1000 chains: 10.4 -> 9.6 ms; ncu: instruction fetch is the largest stall).
+template <int PREC, int NDET, int FORM>
+cudaError_t slice_launch_form(const Model &M, const Tables &T, int slots, const StepArgs &A, cudaStream_t s) {
+    switch (slots) {
+        case 1: k_slice<PREC, NDET, 1, 1, FORM><<<A.k, 32, 0, s>>>(M, T, A); break;
+        case 2: k_slice<PREC, NDET, 2, 2, FORM><<<A.k, 64, 0, s>>>(M, T, A); break;
+        case 4: k_slice<PREC, NDET, 4, 4, FORM><<<A.k, 128, 0, s>>>(M, T, A); break;
+        default: k_slice<PREC, NDET, 8, 8, FORM><<<A.k, 256, 0, s>>>(M, T, A); break;
+    }
+    return cudaGetLastError();
 }
 
 // The work-shared slice update: persistent CTAs (as many as fit on the GPU at
@@ -1333,16 +1331,13 @@ cudaError_t slice_launch(const Model &M, const Tables &T, int slots, const StepA
                 return cudaGetLastError();
             }
         }
-        k_slice<PREC, NDET, 4, 8><<<A.k, 256, 0, s>>>(M, T, A);
+        k_slice<PREC, NDET, 4, 8, FORM_ROT><<<A.k, 256, 0, s>>>(M, T, A);
         return cudaGetLastError();
     }
-    switch (slots) {
-        case 1: k_slice<PREC, NDET, 1><<<A.k, 32, 0, s>>>(M, T, A); break;
-        case 2: k_slice<PREC, NDET, 2><<<A.k, 64, 0, s>>>(M, T, A); break;
-        case 4: k_slice<PREC, NDET, 4><<<A.k, 128, 0, s>>>(M, T, A); break;
-        default: k_slice<PREC, NDET, 8><<<A.k, 256, 0, s>>>(M, T, A); break;
+    if constexpr (PREC == 1) {
+        if (M.tlg >= 5) return slice_launch_form<PREC, NDET, FORM_ROT>(M, T, slots, A, s);
     }
-    return cudaGetLastError();
+    return slice_launch_form<PREC, NDET, FORM_DIRECT>(M, T, slots, A, s);
 }
 
 // Many analyses in one launch (serving), one form of the tiled mixed sums per
