@@ -762,6 +762,9 @@ int ns_init(ns_ctx **out, const ns_prior *prior, const ns_data *data, const ns_p
                     M.pos[dd][i] = data->pos[dd * 3 + i];
                     M.xarm[dd][i] = data->xarm[dd * 3 + i];
                     M.yarm[dd][i] = data->yarm[dd * 3 + i];
+                    M.pos_x[dd][i] = gwns::df_from_double(M.pos[dd][i]);
+                    M.arm_x[2 * dd][i] = gwns::df_from_double(M.xarm[dd][i]);
+                    M.arm_x[2 * dd + 1][i] = gwns::df_from_double(M.yarm[dd][i]);
                 }
     }
     c->d = M.dim;
