@@ -272,13 +272,14 @@ StepArgs step_args(ns_ctx *c, int k) {
     A.active = c->active;
     A.depth = choose_slots(c);
     A.tail = c->n_sm;
-    // FP64 on fine grids: every candidate's bins on two warps, strided by 64, in
-    // every round. A split chosen by the number of chains still running would make
-    // the reduction order, and so the last bits of log L, depend on timing. GB300,
-    // 64,897 / 519,169 bins: the split is 3% / 4% faster than deeper speculation
-    // in the update's tail; on 4017 bins it gains nothing and the extra per-warp
-    // start phasors would cost ~10%.
-    A.fp64_split = (c->precision == NS_FP64 && c->M.model == M_GW && !c->M.rb && c->M.N >= 32768 &&
+    // FP64 above 1024 bins: every candidate's bins on two warps, strided by 64, in
+    // every round (a base depth of two candidates leaves the other two of a chain's
+    // four warps without bins). A split chosen by the number of chains still running
+    // would make the reduction order, and so the last bits of log L, depend on
+    // timing. GB300, slice update of 2000 / 4017 / 16,065 bins (2, 3 and 3 detectors):
+    // 3.60 / 3.67 / 12.6 ms without, 2.71 / 3.40 / 10.2 with the split; 512 bins plan
+    // four candidates for four warps.
+    A.fp64_split = (c->precision == NS_FP64 && c->M.model == M_GW && !c->M.rb && c->M.N > 1024 &&
                     slots_alloc(c) >= 2) ? 2 : 1;
     A.kernel = c->kernel;
     A.walk_scale = c->walk_scale;

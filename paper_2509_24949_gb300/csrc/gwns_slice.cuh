@@ -1018,7 +1018,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             else chain_run(M, A, c, cq, chain, iter, lstar, e_next, e_next_step);
             // plan the base depth while many chains run; the stragglers of the
             // update (fewer running chains than the tail threshold) use every warp.
-            // FP64 on fine grids splits every candidate's bins over two warps in
+            // FP64 above 1024 bins splits every candidate's bins over two warps in
             // every round instead (FP64 branch below), with at most W/2 candidates.
             int depth = S, tail = 1;
             if (A.active) {
@@ -1177,7 +1177,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                 if (dd == 0 && sc < ns && lane < S * NDET) lval[sc] = t - 0.5 * coef[sc].hh;
             }
         } else if (PREC == 0 && W > 1 && M.model == M_GW && !M.rb && tailmode == 2) {
-            // FP64 on fine grids: each candidate's bins on two warps (warps on
+            // FP64 above 1024 bins: each candidate's bins on two warps (warps on
             // different SM sub-partitions issue FP64 independently), bin j on
             // lane j mod 32 of warp (j / 32) mod 2; the two warp sums meet in
             // shared memory in a fixed order, whatever the round.
