@@ -55,11 +55,16 @@ bool is_fin(double x) { return std::isfinite(x); }
 int choose_warps(const ns_ctx *c) {
     if (c->warps > 0) return c->warps;
     if (c->M.model == M_TOY) return 1;
-    // FP64: the FP64 pipe binds, so one warp per point keeps the per-point
-    // overheads lowest once every SM sub-partition has a chain; mixed: more
-    // warps per point hide FP32 latency. Tuned values come from the autotuner.
     const int bins = c->M.N;
-    if (c->precision == NS_FP64) return bins > 32768 ? 2 : 1;
+    // FP64 (k_eval_fx): into how many parts a point's rows are cut, the CTA's four
+    // warps sharing the parts of its points. By the grid alone, so that log L does
+    // not depend on the batch. More parts shorten small batches, whose longest
+    // point binds, and even out the warps; each costs a reduction. GB300, 1 / 2 / 4 / 8
+    // parts: 64 draws of 4017 bins 42.9 / 37.0 / 35.8 / 35.7 us, 8192 draws 104.8 /
+    // 103.4 / 106.7 / 118.9; 64 draws of 16,065 bins 79 / 57 / 43 / 46, 8192 draws 262 /
+    // 238 / 229 / 240; 64 draws of 519,169 bins 259 / 146 / 92 / 91; 8192 draws of 512
+    // bins 52.7 / 54.5 / 59.6 / 68.4.
+    if (c->precision == NS_FP64) return bins <= 1024 ? 1 : (bins <= 8192 ? 2 : 4);
     // the rotation form (tiles of 32 bins or more) prefetches its loads and
     // needs fewer warps per point (GB300, 519,169 bins in 128-bin tiles: 8 / 4 /
     // 2 warps give 1.50 / 1.59 / 1.53 M evals/s). Up to 262,144 bins the batched
