@@ -132,8 +132,19 @@ __device__ __forceinline__ void warp_point_coef(const Model &M, const Tables &T,
 // and there, as for physical-parameter and toy inputs, a CTA takes one point.
 constexpr int EVAL_PPC = 4;
 
+// CTAs per SM that the batched likelihood's kernels are compiled for. Left alone,
+// the compiler settled on 56 to 106 registers, by whatever else the kernel held, and
+// kept too few of the tile loop's loads and chains in flight; 16 warps an SM at 128
+// registers (fewer registers with one detector, whose tile loop needs less) is
+// faster on every grid in tiles of 32 bins or more. GB300, 100 / 8192 draws, before ->
+// now: 3 detectors, 104,000 bins 656 / 1633 -> 478 / 1558 us, 519,169 bins 232 / 4056 ->
+// 200 / 3991; 2 detectors, 31,489 bins 250 / 604 -> 162 / 500; 1 detector, 129,793
+// bins 487 / 1256 -> 387 / 1147.
+#define EVAL_BATCH_BLOCKS(NDET, W) ((NDET) == 1 ? ((W) == 4 ? 5 : 32 / (W)) : 16 / (W))
+#define EVAL_BLOCKS(PREC, NDET, W) ((PREC) == 0 ? 16 / (W) : (NDET) == 1 ? 32 / (W) : (NDET) == 2 ? 20 / (W) : 16 / (W))
+
 template <int PREC, int NDET, int W>
-__global__ void __launch_bounds__(W * 32) k_eval(Model M, Tables T, const double *in, int in_is_theta,
+__global__ void __launch_bounds__(W * 32, EVAL_BLOCKS(PREC, NDET, W)) k_eval(Model M, Tables T, const double *in, int in_is_theta,
                                                  int m, int ppc, double *logl, RunState *st) {
     __shared__ Coef coef[EVAL_PPC];
     __shared__ CoefMixed cm[EVAL_PPC];
@@ -206,7 +217,7 @@ __global__ void __launch_bounds__(W * 32) k_eval(Model M, Tables T, const double
 // of four points on one warp, the other warp waiting, every point's tile groups
 // shared by both warps and reduced in FP64) reached 5.75e7 evals/s.
 template <int NDET, int W>
-__global__ void __launch_bounds__(W * 32) k_eval_batch(Model M, Tables T, const double *in, int m, double *logl,
+__global__ void __launch_bounds__(W * 32, EVAL_BATCH_BLOCKS(NDET, W)) k_eval_batch(Model M, Tables T, const double *in, int m, double *logl,
                                                        RunState *st) {
     constexpr int NG = W >= 2 ? W / 2 : 1;
     constexpr int PPC = 4 * NG;
