@@ -96,10 +96,12 @@ def recorded_traffic():
 
 
 def fp64_flops_per_point_bin(n_det: int) -> float:
-    """Algorithmic FP64 work of one point-bin, in flops (2 per FMA-equivalent):
-    the phase as 8 basis FMAs, one sine/cosine pair (32 FMA-equivalents,
-    measured by instruction count), and per detector the complex product with
-    the weighted data and one Horner step of the detector rotation (8)."""
+    """FP64 work of one point-bin summed bin by bin in FP64 instructions, in flops
+    (2 per FMA-equivalent): the phase as 8 basis FMAs, one sine/cosine pair (32
+    FMA-equivalents), and per detector the complex product with the weighted
+    data and one Horner step of a detector rotation (8). The FP64 form takes
+    neither these instructions nor, on long grids, every bin: its rate in these
+    units says what the FP64 pipe would have to reach."""
     return 2.0 * (8 + 32 + 8 * n_det)
 
 
@@ -275,7 +277,7 @@ def run_gpu(args):
     # the whole run to the stopping rule, from the same initial state
     ttl = time_to_logz_from(sp, blob) if extras else None
     sp.close()
-    # the FP64 form on the same first iteration (one step: ~9 s on this grid)
+    # the FP64 form on the same first iteration (one step)
     fp64 = fp64_first_iteration(g, w, inputs, stream, flush) if extras else None
     # end to end through the C ABI with host buffers
     e2e = e2e_run(g, w, inputs, args.steps, stream)
@@ -387,7 +389,7 @@ def time_to_logz_from(sp, blob):
 
 def fp64_first_iteration(g, w, inputs, stream, flush):
     """The FP64 form on the same grid: its first iteration timed with CUDA
-    events (one step; the FP64 pipe makes it ~40x slower than mixed here)."""
+    events (one step)."""
     import torch
     sp = sampler_on(g, w, inputs, g.NS_FP64, stream)
     blob = sp.checkpoint()
@@ -395,8 +397,9 @@ def fp64_first_iteration(g, w, inputs, stream, flush):
     sp.close()
     t = sum(ms) / 1e3
     return {"evals_per_s": ev / t, "ms_per_step": sum(ms), "evals": ev, "point_bins_per_s": pb / t,
-            "k_slice_frac_fp64_pipe": pb * fp64_flops_per_point_bin(w.n_det) / (kern[3] / 1e3) / (FP64_PEAK_TFLOPS * 1e12),
-            "note": "first iteration, one step, CUDA events; FP64 peak derived (2 FMA/clk/SM)"}
+            "k_slice_fp64_pipe_equivalent": pb * fp64_flops_per_point_bin(w.n_det) / (kern[3] / 1e3) / (FP64_PEAK_TFLOPS * 1e12),
+            "note": "first iteration, one step, CUDA events; the equivalent is the FP64 instructions of a bin-by-bin "
+                    "sum over the FP64 pipe's derived peak (2 FMA/clk/SM): the form runs off that pipe"}
 
 
 def per_point_agreement(g, w, inputs, stream, points=1024):
@@ -801,8 +804,7 @@ def table_row(g, name, precision, stream, max_steps=100000, coarse=False):
     if coarse:
         frac, pipe = None, None     # relative-binning sums, not the per-bin work these counts describe
     elif precision == g.NS_FP64:
-        frac = pb * fp64_flops_per_point_bin(w.n_det) / (slice_ms / 1e3) / (FP64_PEAK_TFLOPS * 1e12)
-        pipe = "FP64"
+        frac, pipe = None, None     # the form reads node rows in place of bins on long grids
     else:
         frac, pipe = mixed_roofline(pb, slice_ms / 1e3, w.n_det, st1["mixed_tile"])
     exe = None
@@ -849,7 +851,8 @@ def batch_eval_row(g, name, precision, stream, points=2048, reps=3, warps=0):
            "point_bins_lo": st1["batch_point_bins_lo"] - st0["batch_point_bins_lo"],
            "batch_evals_per_s": points * reps / t, "point_bins_per_s": pb / t, "bins_per_eval": pb / (points * reps)}
     if precision == g.NS_FP64:
-        row["frac"], row["pipe"] = pb * fp64_flops_per_point_bin(w.n_det) / t / (FP64_PEAK_TFLOPS * 1e12), "FP64"
+        row["frac"], row["pipe"] = None, None
+        row["fp64_pipe_equivalent"] = pb * fp64_flops_per_point_bin(w.n_det) / t / (FP64_PEAK_TFLOPS * 1e12)
     else:
         row["frac"], row["pipe"] = mixed_roofline(pb, t, w.n_det, st1["mixed_tile"])
         row["mixed_tile"] = st1["mixed_tile"]
@@ -905,7 +908,7 @@ def run_table(args):
     for prec in (g.NS_FP64, g.NS_MIXED):
         rows.append(table_row(g, "c4", prec, stream, coarse=True))
     rows.append(table_row(g, "c4", g.NS_MIXED, stream))                  # the whole run (~17 s)
-    rows.append(table_row(g, "c4", g.NS_FP64, stream, max_steps=1))      # one iteration (~9 s)
+    rows.append(table_row(g, "c4", g.NS_FP64, stream, max_steps=1))      # one iteration
     for name in ("c2", "c4"):
         rows.append(batch_eval_row(g, name, g.NS_FP64, stream, points=2048))
         rows.append(batch_eval_row(g, name, g.NS_MIXED, stream, points=8192))
