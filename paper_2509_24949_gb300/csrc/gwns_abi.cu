@@ -521,6 +521,39 @@ static double tile_bound(const double *r, double fc, double h) {
     return best;
 }
 
+// Lagrange polynomials of the nodes at a shortest tile's bins [0] and at a tile's
+// halves' nodes [1], [position][node]: constants, computed in extended precision
+// once per process (0.6 ms where long double is software).
+static const std::vector<double> *lagrange_tables() {
+    static std::vector<double> lag[2];
+    static const bool done = [] {
+        constexpr int n = gwns::FX_NODES;
+        long double y[n];
+        for (int k = 0; k < n; k++) y[k] = std::cos((2 * k + 1) * 3.14159265358979323846264338327950288L / (2 * n));
+        long double den[n];         // 1 / prod_{q != k} (y_k - y_q)
+        for (int k = 0; k < n; k++) {
+            long double v = 1.0L;
+            for (int q = 0; q < n; q++)
+                if (q != k) v *= y[k] - y[q];
+            den[k] = 1.0L / v;
+        }
+        for (int t = 0; t < 2; t++) {
+            lag[t].resize(2 * n * n);
+            for (int i = 0; i < 2 * n; i++) {
+                const long double x = t == 0 ? (i - (n - 0.5L)) / n : 0.5L * (y[i % n] + (i < n ? -1.0L : 1.0L));
+                long double left[n + 1], right[n + 1];     // products of (x - y_q) below and above k
+                left[0] = right[n] = 1.0L;
+                for (int q = 0; q < n; q++) left[q + 1] = left[q] * (x - y[q]);
+                for (int q = n - 1; q >= 0; q--) right[q] = right[q + 1] * (x - y[q]);
+                for (int k = 0; k < n; k++) lag[t][i * n + k] = (double)(left[k] * right[k + 1] * den[k]);
+            }
+        }
+        return true;
+    }();
+    (void)done;
+    return lag;
+}
+
 // The node tiles of a long grid (FxTiles): the box of the phase coefficients from
 // prior draws (with 2% to spare; a point outside it is summed bin by bin), for
 // each tile length the first bin from which the bound above stays below 1e-15
@@ -607,29 +640,8 @@ static int choose_tiles_fx(ns_ctx *c) {
         if (k < NB) r.a[k] = v; else r.t[0] = v;
     }
     r.sh = E + 7;
-    // Lagrange polynomials of the nodes y_n at a shortest tile's bins and at its halves' nodes
     constexpr int n = gwns::FX_NODES;
-    long double y[n];
-    for (int k = 0; k < n; k++) y[k] = std::cos((2 * k + 1) * 3.14159265358979323846264338327950288L / (2 * n));
-    long double den[n];         // 1 / prod_{q != k} (y_k - y_q)
-    for (int k = 0; k < n; k++) {
-        long double v = 1.0L;
-        for (int q = 0; q < n; q++)
-            if (q != k) v *= y[k] - y[q];
-        den[k] = 1.0L / v;
-    }
-    std::vector<double> lag[2];
-    for (int t = 0; t < 2; t++) {
-        lag[t].resize(2 * n * n);
-        for (int i = 0; i < 2 * n; i++) {
-            const long double x = t == 0 ? (i - (n - 0.5L)) / n : 0.5L * (y[i % n] + (i < n ? -1.0L : 1.0L));
-            long double left[n + 1], right[n + 1];     // products of (x - y_q) below and above k
-            left[0] = right[n] = 1.0L;
-            for (int q = 0; q < n; q++) left[q + 1] = left[q] * (x - y[q]);
-            for (int q = n - 1; q >= 0; q--) right[q] = right[q + 1] * (x - y[q]);
-            for (int k = 0; k < n; k++) lag[t][i * n + k] = (double)(left[k] * right[k + 1] * den[k]);
-        }
-    }
+    const std::vector<double> *lag = lagrange_tables();
     const size_t nv = (size_t)((M.N - X.first[0]) >> gwns::FX_LG0) * n * M.n_det;
     if ((rc = dalloc(&c->fx.lag0, 2 * n * n)) || (rc = dalloc(&c->fx.lag1, 2 * n * n)) || (rc = dalloc(&c->fx.v[0], nv)) ||
         (rc = dalloc(&c->fx.v[1], nv / 2 + 1)))
@@ -834,7 +846,12 @@ int ns_init(ns_ctx **out, const ns_prior *prior, const ns_data *data, const ns_p
         c->T.f64 = c->f64;
         if (e == cudaSuccess) e = build_tables(c);
         if (e == cudaSuccess && split) {
-            if ((rc = alloc_fx(c))) { ns_free(c); return rc; }
+            try {
+                rc = alloc_fx(c);
+            } catch (const std::bad_alloc &) {
+                rc = NS_ERR_OOM;
+            }
+            if (rc) { ns_free(c); return rc; }
             e = gwns::launch_fx_sc(c->fx.sc, c->stream);
             if (e == cudaSuccess) e = launch_build_fx(c->M, c->T, c->w64, c->fx, c->stream);
         }
