@@ -746,6 +746,7 @@ int ns_init(ns_ctx **out, const ns_prior *prior, const ns_data *data, const ns_p
         }
         M.dim = dim;
         M.inv_df = 1.0 / M.df;
+        M.cut32 = (M.f0 + (double)M.N * M.df) * M.inv_df <= (double)(1 << 22);
         // periodic parameters -> unit-cube coordinates
         M.periodic = 0;
         for (int p = 0, i = 0; p < NS_NPARAM; p++) {

@@ -51,6 +51,7 @@ struct Model {
     int np;           // tiled form: N padded to whole groups of 32 tiles
     double f0, df;
     double inv_df;    // 1 / df
+    int cut32;        // 1: the cutoff index may be guessed in FP32 (cutoff_index_tab)
     int kind[NPARAM];
     double lo[NPARAM], hi[NPARAM];
     double pbase[NPARAM], pspan[NPARAM];   // uniform: lo, hi - lo; volume: lo^3, hi^3 - lo^3
@@ -273,15 +274,18 @@ __device__ __forceinline__ void prior_transform(const Model &M, const double *u,
 // Last grid index with f_j <= fisco, in [-1, N-1], from the grid's frequency
 // table (f64[j] holds the rounded f0 + j*df the tables use): a first guess by
 // one multiplication, then at most a few steps either way against the table. The
-// guess is in FP32 where that is within a bin or so, the comparisons are of the
-// bit patterns (positive doubles order as their bits do): FP64 instructions cost
-// 64 cycles each. A NaN or a fisco that is not positive gives -1.
+// guess is in FP32 on grids that end below 2^22 df (Model::cut32), the comparisons
+// are of the bit patterns (positive doubles order as their bits do): FP64
+// instructions cost 64 cycles each. With a highest frequency F the FP32 guess is off
+// by the roundings of fisco, f0, their difference, 1/df and the product, at most
+// 5 F 2^-24 / df bins: 1.25 at F = 2^22 df, which the steps cover; it grows with
+// F / df whatever the number of bins. A NaN or a fisco that is not positive gives -1.
 __device__ __forceinline__ int cutoff_index_tab(const Model &M, const double *f64, double fisco) {
     if (!M.cutoff) return M.N - 1;
     const long long fb = __double_as_longlong(fisco);
     if (fb <= 0 || fb > 0x7ff0000000000000ll) return -1;
     int j;
-    if (M.N <= (1 << 20)) {
+    if (M.cut32) {
         const float g = ((float)fisco - (float)M.f0) * (float)M.inv_df;
         j = g < -1.0f ? -1 : g > (float)(M.N - 1) ? M.N - 1 : (int)floorf(g);
     } else {
