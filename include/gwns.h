@@ -62,8 +62,9 @@ enum { NS_PRIOR_FIXED = 0, NS_PRIOR_UNIFORM = 1, NS_PRIOR_VOLUME = 2 };
 /* Inner kernels of the update (ns_options.kernel). */
 enum { NS_KERNEL_SLICE = 0, NS_KERNEL_WALK = 1 };
 /* Arithmetic of the likelihood (ns_options.precision). NS_FP64: to FP64 accuracy
- * (coefficients in FP64; per-bin phases in 58-bit fixed point, products and sums in
- * double-float, all nearer to the exact sum than FP64 instructions are on long grids).
+ * (coefficients in FP64; per-bin phases in 60-bit fixed point, rounded below FP64's at
+ * every frequency; products and sums in double-float, about 48 bits. Together the sums
+ * over bins are no further from the exact ones than FP64 instructions make them).
  * NS_MIXED: per-point coefficients in double-float (pairs of floats on the FP32
  * pipe; the FP64 stage instead when the environment variable GWNS_COEF_FP64=1 is
  * set at ns_init, or for relative binning), the per-bin phase in double-float,

@@ -9,6 +9,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <tuple>
@@ -134,19 +135,19 @@ int capture_iteration(ns_ctx *c, int k) {
     return NS_OK;
 }
 
-// The binary exponents that bring the basis functions and the frequency below
-// one on the grid: each is monotone there but f^(1/3) ln f, whose minimum is -3/e
-// at f = e^-3.
-void fx_exponents(ns_ctx *c) {
+// Half-width of the delays t_c + dt_d about the middle of the t_c prior: its
+// half-range plus the largest light travel time to the geocentre.
+double delay_radius(const Model &M) {
+    double rmax = 0.0;
+    if (!M.ideal)
+        for (int d = 0; d < M.n_det; d++)
+            rmax = std::max(rmax, std::sqrt(M.pos[d][0] * M.pos[d][0] + M.pos[d][1] * M.pos[d][1] + M.pos[d][2] * M.pos[d][2]));
+    return 0.5 * (M.hi[P_TC] - M.lo[P_TC]) + rmax / gwns::C_SI;
+}
+
+void make_blocks(ns_ctx *c) {
     const Model &M = c->M;
-    double mx[NB + 1] = {};
-    for (const double f : {M.f0, M.f0 + (double)(M.N - 1) * M.df}) {
-        const double r = std::cbrt(f), l = std::log(f);
-        const double B[NB + 1] = {1.0 / (f * r * r), 1.0 / f, 1.0 / (r * r), 1.0 / r, l, r, r * l, r * r, f};
-        for (int m = 0; m <= NB; m++) mx[m] = std::max(mx[m], std::fabs(B[m]));
-    }
-    mx[6] = std::max(mx[6], 1.2);
-    for (int m = 0; m <= NB; m++) c->T.fxe[m] = std::ilogb(std::max(mx[m] * (1.0 + 1e-12), 1e-300)) + 1;
+    gwns::fx_make_blocks(M.N, M.f0, M.df, M.lo[P_MC], 0.5 * delay_radius(M), c->T.tiles, c->T.fxk);
 }
 
 // Relative-binning tables for the current data (edges, fiducial coefficients,
@@ -173,6 +174,8 @@ int build_rb(ns_ctx *c) {
              (rc = dalloc(&X.hs, nd)) || (rc = dalloc(&c->fx.sc, gwns::FX_SC))))
             return rc;
     }
+    std::unique_ptr<int[]> J(new (std::nothrow) int[ne]);
+    if (!J) return NS_ERR_OOM;
     double2 *h0 = nullptr;
     double *th = nullptr;
     if ((rc = dalloc(&h0, (size_t)nd * c->M.N)) || (rc = dalloc(&th, NS_NPARAM))) { dfree(h0); return rc; }
@@ -187,6 +190,7 @@ int build_rb(ns_ctx *c) {
                             c->rb_A1, c->rb_B0, c->rb_B1, c->rb_A0f, c->rb_A1f, c->rb_B0f, c->rb_B1f,
                             c->rb_inv_de_f, c->stream);
     int nedge = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(J.get(), c->rb_J, sizeof(int) * ne, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&nedge, c->rb_nedge, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(h0);
@@ -201,7 +205,10 @@ int build_rb(ns_ctx *c) {
     T.inv_de_f = c->rb_inv_de_f; T.fid = c->rb_fid;
     if (c->precision == NS_FP64) {
         const gwns::RBFx &X = c->rb_fx;
-        fx_exponents(c);
+        // the grid's blocks of frequency, counted in edges
+        make_blocks(c);
+        gwns::FxBlocks &K = c->T.fxk;
+        for (int b = 0; b < K.n; b++) K.bin[b] = (int)(std::lower_bound(J.get(), J.get() + nedge, K.bin[b]) - J.get());
         CK(gwns::launch_fx_sc(c->fx.sc, c->stream));
         CK(gwns::launch_rb_fx(c->M, c->T, T, X, c->stream));
         c->T.fxsc = c->fx.sc;
@@ -585,13 +592,8 @@ static int choose_tiles_fx(ns_ctx *c) {
         ba[k] = 0.5 * (lo + hi);
         br[k] = 0.51 * (hi - lo) + 1e-9 * std::max(std::fabs(lo), std::fabs(hi));
     }
-    // delays: t_c plus the light travel time to the geocentre
-    double rmax = 0.0;
-    if (!M.ideal)
-        for (int d = 0; d < M.n_det; d++)
-            rmax = std::max(rmax, std::sqrt(M.pos[d][0] * M.pos[d][0] + M.pos[d][1] * M.pos[d][1] + M.pos[d][2] * M.pos[d][2]));
     ba[NB] = 0.5 * (M.lo[P_TC] + M.hi[P_TC]);
-    br[NB] = (0.5 * (M.hi[P_TC] - M.lo[P_TC]) + rmax / gwns::C_SI) * (1.0 + 1e-9) + 1e-12;
+    br[NB] = delay_radius(M) * (1.0 + 1e-9) + 1e-12;
     if (!std::isfinite(ba[NB]) || !std::isfinite(br[NB])) return NS_OK;
     int rows = M.N;
     for (int l = 0; l < gwns::FX_LEV; l++) {
@@ -625,21 +627,6 @@ static int choose_tiles_fx(ns_ctx *c) {
         return NS_OK;
     }
     c->fx.n = rows;
-    // the reference point: the box's centre
-    gwns::FxPoint &r = c->fx.ref;
-    std::memset(&r, 0, sizeof(r));
-    uint64_t mant[NB + 1];
-    int ex[NB + 1], E = 0, bad = 0;
-    for (int k = 0; k <= NB; k++) {
-        ex[k] = (k < NB ? gwns::fx_mantissa<true>(ba[k], &mant[k], &bad) : gwns::fx_mantissa<false>(ba[k], &mant[k], &bad))
-              + c->T.fxe[k] + 64;
-        E = std::max(E, ex[k]);
-    }
-    for (int k = 0; k <= NB; k++) {
-        const gwns::fx2 v = gwns::fx_split(gwns::fx_scaled(mant[k], E - ex[k] + 6, ba[k]));
-        if (k < NB) r.a[k] = v; else r.t[0] = v;
-    }
-    r.sh = E + 7;
     constexpr int n = gwns::FX_NODES;
     const std::vector<double> *lag = lagrange_tables();
     const size_t nv = (size_t)((M.N - X.first[0]) >> gwns::FX_LG0) * n * M.n_det;
@@ -657,10 +644,14 @@ static int choose_tiles_fx(ns_ctx *c) {
 static int alloc_fx(ns_ctx *c) {
     const Model &M = c->M;
     const size_t nd = M.n_det;
-    fx_exponents(c);
     c->fx.n = M.N;
     int rc = choose_tiles_fx(c);
     if (rc) return rc;
+    make_blocks(c);
+    const gwns::FxBlocks &K = c->T.fxk;
+    // the tiles' reference point: the box's centre
+    int32_t bad = 0;
+    for (int b = 0; b < K.n; b++) gwns::fx_coef(K, b, c->T.box_a, c->T.box_a + NB, 1, 0.0, c->fx.ref[b], bad);
     const size_t rows = c->fx.n;
     if ((rc = dalloc(&c->fx.b, NB / 2 * rows)) || (rc = dalloc(&c->fx.f, rows)) ||
         (rc = dalloc(&c->fx.w, nd * rows)) || (rc = dalloc(&c->fx.scale, nd)) || (rc = dalloc(&c->fx.wmax, nd)) ||

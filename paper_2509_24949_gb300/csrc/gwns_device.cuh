@@ -109,7 +109,7 @@ struct Tables {
     FxTiles tiles;           // node rows after the bins' (long grids)
     // the points that the tiles serve: |a_m - box_a[m]| <= box_r[m], |tau_d - box_a[NB]| <= box_r[NB]
     double box_a[NB + 1], box_r[NB + 1];
-    int fxe[NB + 1];         // binary exponents of the basis functions' and the frequency's scale
+    FxBlocks fxk;            // blocks of frequency with the exponents of their tables' scales
     const double *prefix;    // [n_det][N] P_d(j)
     // mixed form, per bin (Model::tlg == 0)
     const float2 *basis32;   // [NB][N]   B_m(f_j) as (hi, lo) floats
@@ -830,7 +830,7 @@ __device__ __forceinline__ void sincos_bf(double x, double &s, double &c) {
 }
 
 // FP64 form: the coefficients of up to four points as fixed-point integers on
-// one scale per point (gwns_fx.cuh): lane group g (8 lanes) takes point g, its
+// one scale per point and block of frequency (gwns_fx.cuh): lane group g (8 lanes) takes point g, its
 // sub-lane m basis coefficient m, then detector m's delay and (sub-lane 0) the
 // constant phase. Integer instructions only. All 32 lanes must call.
 // With fid, the differences from the fiducial point's coefficients.
@@ -849,29 +849,42 @@ __device__ inline void coef_to_fx_group(const Tables &T, int n_det, const Coef *
         tau -= fid->tau[det ? sl : 0];
         ph -= fid->c0u;
     }
-    const int ea = fx_mantissa<true>(a, &ma, &bad) + T.fxe[sl];
-    const int et = fx_mantissa<false>(tau, &mt, &bad) + T.fxe[NB];
-    const int ec = fx_mantissa<true>(ph, &mc, &bad);
+    const int xa = fx_mantissa<true>(a, &ma, &bad) + 64, xt = fx_mantissa<false>(tau, &mt, &bad) + 64;
+    const int ec = fx_mantissa<true>(ph, &mc, &bad) + 64;
     // inside the tiles' box? (a NaN is not)
     bool in = true;
     if (T.tiles.nlev > 0)
         in = fabs(a - T.box_a[sl]) <= T.box_r[sl] && (!det || fabs(tau - T.box_a[NB]) <= T.box_r[NB]);
     in = ((__ballot_sync(0xffffffffu, in) >> (lane & 24)) & 0xffu) == 0xffu;
-    // the point's scale 2^E: above every term's largest value on the grid
-    int E = max(max(max(ea, et), ec) + 64, 0);
+#pragma unroll 1
+    for (int b = 0; b < T.fxk.n; b++) {
+        const int ea = xa + T.fxk.e[b][sl], et = xt + T.fxk.e[b][NB];
+        // the point's scale 2^E: above every term's largest value in the block
+        int E = max(max(max(ea, et), ec), 0);
 #pragma unroll
-    for (int w = 4; w > 0; w >>= 1) {
-        E = max(E, __shfl_xor_sync(0xffffffffu, E, w, 8));
-        bad |= __shfl_xor_sync(0xffffffffu, bad, w, 8);
+        for (int w = 4; w > 0; w >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, w, 8));
+        if (!writer) continue;
+        FxCoef &q = o.blk[b];
+        q.a[sl] = fx_split(fx_scaled(ma, fx_shift(E, ea), a));
+        if (det) q.t[sl] = fx_split(fx_scaled(mt, fx_shift(E, et), tau));
+        if (sl == 0) {
+            q.c0 = fx_scaled(mc, fx_shift(E, ec) + 1, ph);
+            q.sh = fx_lift(E);
+            // without tiles a row is a bin
+            q.end = b + 1 < T.fxk.n ? T.fxk.bin[b + 1] : 0x7fffffff;
+        }
     }
-    if (!writer) return;
-    o.a[sl] = fx_split(fx_scaled(ma, E - (ea + 64) + 6, a));
-    if (det) o.t[sl] = fx_split(fx_scaled(mt, E - (et + 64) + 6, tau));
-    if (sl == 0) {
-        o.c0 = fx_scaled(mc, E - (ec + 64) + 7, ph);
-        o.sh = E + 7;
+    bad = (__ballot_sync(0xffffffffu, bad) >> (lane & 24)) & 0xffu;
+    if (writer && sl == 0) {
         o.bad = bad;
-        fx_segments(T.tiles, in, c.jcut + 1, o);
+        if (T.tiles.nlev > 0) {
+            fx_layout(T.tiles, &T.fxk, in, c.jcut + 1, o);
+        } else {
+            o.nseg = 1;
+            o.rows = c.jcut + 1;
+            o.seg[0].end = 0x7fffffff;
+            o.seg[0].off = 0;
+        }
     }
 }
 
@@ -880,6 +893,39 @@ __device__ inline void coef_to_fx_group(const Tables &T, int n_det, const Coef *
 __device__ __forceinline__ void load_sc(const Tables &T, float4 *sc) {
     for (int i = threadIdx.x; i < FX_SC; i += blockDim.x) sc[i] = __ldg(T.fxsc + i);
 }
+
+// A point's coefficients in one block, in registers.
+template <int NDET>
+struct FxRegs {
+    fx2 a[NB], t[NDET];
+    int64_t c0;
+    int32_t sh;
+    __device__ __forceinline__ explicit FxRegs(const FxCoef &c) { load(c); }
+    __device__ __forceinline__ void load(const FxCoef &c) {
+#pragma unroll
+        for (int m = 0; m < NB; m++) a[m] = c.a[m];
+#pragma unroll
+        for (int d = 0; d < NDET; d++) t[d] = c.t[d];
+        c0 = c.c0;
+        sh = c.sh;
+    }
+    // the constant's and the basis terms' sums at table row b (N rows)
+    __device__ __forceinline__ void basis(const int4 *b, int N, int64_t &hi, int64_t &cr) const {
+        hi = c0;
+        cr = FX_HALF;
+#pragma unroll
+        for (int m = 0; m < NB; m += 2) {
+            const int4 v = __ldg(b + (size_t)(m >> 1) * N);
+            fx_mac(hi, cr, a[m], fx2{v.x, v.y});
+            fx_mac(hi, cr, a[m + 1], fx2{v.z, v.w});
+        }
+    }
+    // detector d's phase at frequency f
+    __device__ __forceinline__ uint64_t phase(int64_t hi, int64_t cr, int d, int2 f) const {
+        fx_mac(hi, cr, t[d], fx2{f.x, f.y});
+        return fx_phase(hi, cr, sh);
+    }
+};
 
 // FP64 form: Z_d = sum_j w_dj exp(i Psi_dj) over the point's rows j0, j0 + stride, ..
 // in the split arithmetic of gwns_fx.cuh, each detector's phase by its own
@@ -899,31 +945,27 @@ __device__ __forceinline__ void bins_fx(const Tables &T, const FxPoint &c, const
         zl[d][0] = zl[d][1] = 0.f;
     }
     if (c.bad) return;
-    fx2 a[NB], t[NDET];
-#pragma unroll
-    for (int m = 0; m < NB; m++) a[m] = c.a[m];
-#pragma unroll
-    for (int d = 0; d < NDET; d++) t[d] = c.t[d];
-    const int64_t c0 = c.c0;
-    const int32_t sh = c.sh;
-    int seg = 0;
+    FxRegs<NDET> q(c.blk[0]);
+    int seg = 0, blk = 0, lim = 0, off = 0;     // rows up to lim lie in this segment and block
 #pragma unroll 1
     for (int r = j0; r < rows; r += stride) {
-        while (r >= c.seg[seg].end) seg++;
-        const int j = r + c.seg[seg].off;
-        int64_t hi = c0, cr = 0;
-#pragma unroll
-        for (int m = 0; m < NB; m += 2) {
-            const int4 b = __ldg(T.fxb + (size_t)(m >> 1) * N + j);
-            fx_mac(hi, cr, a[m], fx2{b.x, b.y});
-            fx_mac(hi, cr, a[m + 1], fx2{b.z, b.w});
+        if (r >= lim) {
+            while (r >= c.seg[seg].end) seg++;
+            off = c.seg[seg].off;
+            if (r >= c.blk[blk].end) {
+                do blk++;
+                while (r >= c.blk[blk].end);
+                q.load(c.blk[blk]);
+            }
+            lim = min(c.seg[seg].end, c.blk[blk].end);
         }
+        const int j = r + off;
+        int64_t hi, cr;
+        q.basis(T.fxb + j, N, hi, cr);
         const int2 f = __ldg(T.fxf + j);
 #pragma unroll
         for (int d = 0; d < NDET; d++) {
-            int64_t hd = hi, cd = cr;
-            fx_mac(hd, cd, t[d], fx2{f.x, f.y});
-            const fxe E = fx_cis(fx_phase(hd, cd, sh), sc);
+            const fxe E = fx_cis(q.phase(hi, cr, d, f), sc);
             fx_cmac(zh[d], zl[d], __ldg(T.fxw + (size_t)d * N + j), E);
         }
     }
@@ -1648,8 +1690,9 @@ __device__ __forceinline__ void warp_sum_df_many(float (&h)[16], float (&l)[16],
 // against 11,000 for the FP64 sines, cosines and sums. GB300, 8192 draws on 1024
 // coarse bins: 2.81 ms -> 237 us.
 template <int NDET>
-__device__ __forceinline__ double rb_loglike_fx(const Model &M, const RBTables &R, const Coef &c, const FxPoint &fx,
+__device__ __forceinline__ double rb_loglike_fx(const Model &M, const Tables &T, const Coef &c, const FxPoint &fx,
                                                 const float4 *sc) {
+    const RBTables &R = T.rb;
     const int lane = threadIdx.x & 31;
     // bins whose centre lies at or below f_ISCO: a 32-way search (the centres ascend)
     int nbu = R.nb;
@@ -1673,23 +1716,23 @@ __device__ __forceinline__ double rb_loglike_fx(const Model &M, const RBTables &
     }
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     const int ne = R.nedge;
+    FxRegs<NDET> q(fx.blk[0]);
+    int blk = 0;
 #pragma unroll 1
     for (int base = 0; base < nbu && !fx.bad; base += 31) {
         const int e = min(base + lane, nbu);
         const bool own = lane < 31 && base + lane < nbu, last = base + lane == nbu;
-        int64_t hi = fx.c0, cr = 0;
-#pragma unroll
-        for (int m = 0; m < NB; m += 2) {
-            const int4 b = __ldg(R.fxb + (size_t)(m >> 1) * ne + e);
-            fx_mac(hi, cr, fx.a[m], fx2{b.x, b.y});
-            fx_mac(hi, cr, fx.a[m + 1], fx2{b.z, b.w});
+        if (blk + 1 < T.fxk.n && e >= T.fxk.bin[blk + 1]) {
+            do blk++;
+            while (blk + 1 < T.fxk.n && e >= T.fxk.bin[blk + 1]);
+            q.load(fx.blk[blk]);
         }
+        int64_t hi, cr;
+        q.basis(R.fxb + e, ne, hi, cr);
         const int2 f = __ldg(R.fxf + e);
 #pragma unroll
         for (int d = 0; d < NDET; d++) {
-            int64_t hd = hi, cd = cr;
-            fx_mac(hd, cd, fx.t[d], fx2{f.x, f.y});
-            const fxe E = fx_cis(fx_phase(hd, cd, fx.sh), sc);
+            const fxe E = fx_cis(q.phase(hi, cr, d, f), sc);
             const float4 *gp = (last ? R.GR : R.G) + (size_t)d * ne + e;
             const float4 w = own || last ? __ldg(gp) : zero;
             fx_acc(vh[3 * d], vl[3 * d], w.x, w.y, E.rh, E.rl);

@@ -5,19 +5,33 @@
 // thousands of cycles in FP64 and a few hundred in the split arithmetic here:
 //
 //  * the phase in turns as a fixed-point sum of products, modulo one turn. The
-//    basis and the frequency are 59-bit integers scaled to their largest value
-//    on the grid, a point's coefficients 58-bit integers on one scale per point
-//    (block floating point: unit 2^-58 of the point's largest term, 32 times
-//    finer than FP64's rounding of that term). Both are split into 30-bit
-//    halves, so that the high and the cross products add up in two 64-bit
-//    accumulators without carries: three multiply-adds per term.
+//    grid is cut into blocks of frequency where the phases have fallen far enough
+//    (FxBlocks). In a block the basis and the frequency are 59-bit integers scaled
+//    to their largest value there, a point's coefficients 60-bit integers on one
+//    scale per point and block: the unit is 2^-59 of the power of two above the
+//    point's largest term in the block, where FP64 rounds that term at 2^-53, so
+//    that also a block's last bins are rounded below FP64's sums (0.01 to 0.5 of their rms,
+//    by octave). One scale for a whole grid would give every bin the rounding of
+//    the lowest frequency's terms: rms error of the phases at 50 to 400 Hz, chirp
+//    mass 1.2, grid from 20 / 5 / 1 / 0.1 Hz, FP64 1.3e-13 rad, one scale with
+//    58-bit coefficients and floored halves 5e-13 / 7e-12 / 1.2e-10 / 3.9e-9, blocks
+//    1.0e-13 (the tabulated basis' own rounding).
+//    Both factors are split at 2^30 into a high half and a signed low half, so that
+//    the high and the cross products add up in two 64-bit accumulators without
+//    carries: three multiply-adds per term; the dropped low products average to
+//    nothing (with low halves that are never negative they would shift every
+//    bin's phase the same way).
 //  * exp(2 pi i phase): the top 10 fraction bits pick cos and sin of k 2 pi/1024
 //    from a table (double-float, half a turn, the other half by sign), the rest
 //    r, |r| < 0.0031 rad, enters through sin r and cos r - 1 by their Taylor
 //    polynomials and one complex product, all in double-float (absolute error
 //    about 1e-15).
 //  * the products with the weighted data and their sums in double-float
-//    (48 bits), the data scaled by a power of two per detector.
+//    (48 bits), the data scaled by a power of two per detector. With the phases'
+//    finer rounding the sums as a whole are no further from the exact ones than
+//    an FP64 loop's (rms error over the weights' norm, FP64 -> here, 512 bins
+//    1.6e-14 -> 1.3e-14, 4017 1.4e-14 -> 0.9e-14, low masses on 64,897 bins
+//    1.6e-12 -> 1.0e-12).
 //
 // Plain C++ besides the qualifiers, so the same code compiles for the host
 // (where a CPU test checks it against 60-digit references) and for sm_103a.
@@ -28,27 +42,43 @@ namespace gwns {
 
 constexpr int FX_NB = 8;            // phase basis functions
 constexpr int FX_DET = 4;           // detectors at most
-constexpr int FX_ABITS = 58;        // coefficients: |A| < 2^58
+constexpr int FX_ABITS = 60;        // coefficients: |A| <= 2^60
 constexpr int FX_BBITS = 59;        // tables: |b| <= 2^59
 constexpr int FX_SC = 512;          // table points over half a turn
 constexpr int FX_NODES = 32;        // nodes of a tile (below)
 constexpr int FX_LG0 = 6;           // log2 of the shortest tile's bins
 constexpr int FX_LEV = 10;          // tile levels at most
 constexpr int FX_SEG = 2 * FX_LEV + 1;
+constexpr int FX_BLK = 6;           // blocks of frequency at most
+constexpr int64_t FX_HALF = 1 << 29;    // the cross products' sum starts here: fx_phase rounds
 
-// A signed 60-bit integer as 2^30 h + l, 0 <= l < 2^30.
+// A signed integer of up to 61 bits as 2^30 h + l, -2^29 <= l < 2^29.
 struct fx2 {
     int32_t h, l;
 };
 
-// One point's fixed-point phase coefficients (a: basis, t: detector delays) in
-// units of 2^(E - 58) turns per full-scale table entry; c0 in the phase sum's
-// unit 2^(E - 57) turns; sh = E + 7 lifts the sum's fraction to 64 bits.
-struct FxPoint {
+// Blocks of frequency: block b starts at bin (relative binning: at edge) bin[b],
+// and e[b] are the binary exponents that bring its basis functions and
+// frequencies below one.
+struct FxBlocks {
+    int32_t n;
+    int32_t bin[FX_BLK];
+    int32_t e[FX_BLK][FX_NB + 1];
+};
+
+// One point's fixed-point phase coefficients in a block (a: basis, t: detector
+// delays) in units of 2^(E - 60) turns per full-scale table entry, 2^E the power
+// of two above its largest term; c0 in the phase sum's unit 2^(E - 59) turns;
+// sh = E + 5 lifts the sum's fraction to 64 bits; end: the running row that the
+// block ends at.
+struct FxCoef {
     fx2 a[FX_NB];
     fx2 t[FX_DET];
     int64_t c0;
-    int32_t sh;
+    int32_t sh, end;
+};
+struct FxPoint {
+    FxCoef blk[FX_BLK];
     int32_t bad;        // a coefficient is not finite: the sums are NaN
     // the rows to sum: running index r < rows lies in the first segment with
     // r < end and is table row r + off
@@ -72,7 +102,10 @@ struct fxe {
     float rh, rl, ih, il;       // double-float complex
 };
 
-DFI fx2 fx_split(int64_t v) { return fx2{(int32_t)(v >> 30), (int32_t)(v & 0x3fffffff)}; }
+DFI fx2 fx_split(int64_t v) {
+    const int64_t h = (v + FX_HALF) >> 30;
+    return fx2{(int32_t)h, (int32_t)(v - (h << 30))};
+}
 
 #if defined(__CUDA_ARCH__)
 DFI uint64_t fx_mulhi(uint64_t a, uint64_t b) { return __umul64hi(a, b); }
@@ -102,6 +135,11 @@ DFI int64_t fx_scaled(uint64_t m, int s, double x) {
     return (fx_bits(x) >> 63) ? -(int64_t)v : (int64_t)v;
 }
 
+// The shifts of a coefficient's mantissa (|x| < 2^ex) to the unit 2^(E - FX_ABITS), of
+// the constant phase's (one more) and of the phase sum's fraction to 2^-64 turns.
+DFI int fx_shift(int E, int ex) { return E - ex + 64 - FX_ABITS; }
+DFI int fx_lift(int E) { return E + 65 - FX_ABITS; }
+
 // Table entry of a double with |v| <= 2^eb.
 #if defined(__CUDACC__)
 __device__ __forceinline__ fx2 fx_table(double v, int eb) {
@@ -111,13 +149,31 @@ __device__ __forceinline__ fx2 fx_table(double v, int eb) {
 DFI fx2 fx_table(double v, int eb) { return fx_split(llrint(scalbn(v, FX_BBITS - eb))); }
 #endif
 
+// Block of bin j.
+DFI int fx_block(const FxBlocks &K, int j) {
+    int b = 0;
+    while (b + 1 < K.n && j >= K.bin[b + 1]) b++;
+    return b;
+}
+// Ends of the blocks that a segment closes: bins [pos, e) by units of 2^lg bins
+// with rpt rows each from running row `rows` on. A unit belongs to the block of its
+// first bin.
+DFI void fx_block_ends(const FxBlocks *K, FxPoint &o, int &b, int pos, int e, int lg, int rpt, int rows) {
+    for (int it = 0; K && it < FX_BLK && b + 1 < K->n && K->bin[b + 1] < e; it++) {
+        const int d = K->bin[b + 1] > pos ? K->bin[b + 1] - pos : 0;
+        o.blk[b++].end = rows + ((d + (1 << lg) - 1) >> lg) * rpt;
+    }
+}
+
 // The segments of the bins 0 .. n - 1: bins below the first tiled one, then tiles
 // of growing length, each level up to the next one's first bin, then of
-// shrinking length up to the cutoff and the last few bins one by one.
-DFI void fx_segments(const FxTiles &T, bool tiles, int n, FxPoint &o) {
-    int ns = 0, rows = 0, pos = 0;
+// shrinking length up to the cutoff and the last few bins one by one. With K also
+// the running rows that the blocks end at.
+DFI void fx_layout(const FxTiles &T, const FxBlocks *K, bool tiles, int n, FxPoint &o) {
+    int ns = 0, rows = 0, pos = 0, b = 0;
     if (tiles && T.nlev > 0 && n > T.first[0]) {
         if (T.first[0] > 0) {
+            fx_block_ends(K, o, b, 0, T.first[0], 0, 1, 0);
             pos = rows = T.first[0];
             o.seg[ns].end = rows;
             o.seg[ns++].off = 0;
@@ -132,6 +188,7 @@ DFI void fx_segments(const FxTiles &T, bool tiles, int n, FxPoint &o) {
                 up = true;
             }
             if (e > pos) {
+                fx_block_ends(K, o, b, pos, e, lg, FX_NODES, rows);
                 o.seg[ns].off = T.row[l] + ((pos - T.first[l]) >> lg) * FX_NODES - rows;
                 rows += ((e - pos) >> lg) * FX_NODES;
                 o.seg[ns++].end = rows;
@@ -142,17 +199,90 @@ DFI void fx_segments(const FxTiles &T, bool tiles, int n, FxPoint &o) {
         }
     }
     if (n > pos) {
+        fx_block_ends(K, o, b, pos, n, 0, 1, rows);
         o.seg[ns].off = pos - rows;
         rows += n - pos;
         o.seg[ns++].end = rows;
     }
+    if (K) o.blk[b].end = 0x7fffffff;
     o.nseg = ns;
     o.rows = rows;
 }
+DFI void fx_segments(const FxTiles &T, bool tiles, int n, FxPoint &o) { fx_layout(T, nullptr, tiles, n, o); }
+
+// The blocks of a grid. FP64 rounds a bin's phase by its size there, about the
+// Newtonian term 3/128 (pi T_sun Mc f)^(-5/3) (at the prior's lowest chirp mass mc)
+// plus 2 pi f tau (tau a typical delay) plus 10 rad for the rest; the split
+// arithmetic rounds it by the block's largest term at 2^-5 to 2^-6 of that. So a
+// block ends where the phases have fallen to 1/40 of its first bin's Newtonian term
+// (a larger fall only where FX_BLK blocks do not suffice, on more than five decades of
+// frequency). From 20 Hz, chirp masses of 10 or more take one block, of 1.1 or more two.
+// A block's largest values are taken over its bins and the tiles that start in it,
+// whose nodes reach half a bin beyond the tile's bins. Every basis function is
+// monotone between its ends but f^(1/3) ln f, whose minimum is -3/e at f = e^-3.
+inline void fx_make_blocks(int N, double f0, double df, double mc, double tau, const FxTiles &T, FxBlocks &K) {
+    const double f1 = f0 + (double)(N - 1) * df;
+    auto newton = [&](double f) { return 3.0 / 128.0 * pow(3.141592653589793 * 4.925490947641267e-6 * mc * f, -5.0 / 3.0); };
+    double fall = 40.0;
+    for (int it = 0; it < 64; it++, fall *= 1.5) {
+        K.n = 1;
+        K.bin[0] = 0;
+        int more = 0;
+        double top = newton(f0);
+        for (double f = f0; f < f1; f *= 1.09) {
+            if (!(top > fall * (newton(f) + 6.283185307179586 * f * tau + 10.0))) continue;
+            const double j = ceil((f - f0) / df);
+            if (!(j < (double)N)) break;
+            top = newton(f);
+            if ((int)j <= K.bin[K.n - 1]) continue;
+            if (K.n == FX_BLK) { more = 1; break; }
+            K.bin[K.n++] = (int)j;
+        }
+        if (!more) break;
+    }
+    for (int b = 0; b < K.n; b++) {
+        const int last = (b + 1 < K.n ? K.bin[b + 1] : N) - 1;
+        double lo = f0 + (double)K.bin[b] * df, hi = f0 + (double)last * df;
+        for (int l = 0; l < T.nlev; l++) {
+            const int lg = FX_LG0 + l;
+            if (last < T.first[l]) continue;
+            int end = ((((last - T.first[l]) >> lg) + 1) << lg) + T.first[l];
+            if (end > N) end -= 1 << lg;
+            hi = fmax(hi, f0 + ((double)end - 0.5) * df);
+            if (lo > 8.0 * df) lo = fmin(lo, f0 + ((double)K.bin[b] - 0.5) * df);
+        }
+        double mx[FX_NB + 1] = {};
+        for (int i = 0; i < 2; i++) {
+            const double f = i == 0 ? lo : hi, r = cbrt(f), l = log(f);
+            const double B[FX_NB + 1] = {1.0 / (f * r * r), 1.0 / f, 1.0 / (r * r), 1.0 / r, l, r, r * l, r * r, f};
+            for (int m = 0; m <= FX_NB; m++) mx[m] = fmax(mx[m], fabs(B[m]));
+        }
+        if (lo < 0.05 && hi > 0.049) mx[6] = fmax(mx[6], 1.2);
+        for (int m = 0; m <= FX_NB; m++) K.e[b][m] = ilogb(fmax(mx[m] * (1.0 + 1e-12), 1e-300)) + 1;
+    }
+}
+
+// A point's coefficients in block b from its basis coefficients a [rad], delays
+// tau [s] and constant phase c0 [rad]; bad is set where one is not finite.
+inline void fx_coef(const FxBlocks &K, int b, const double *a, const double *tau, int nt, double c0, FxCoef &o,
+                    int32_t &bad) {
+    uint64_t m[FX_NB + FX_DET + 1];
+    int ex[FX_NB + FX_DET + 1], E = 0;
+    for (int i = 0; i < FX_NB; i++) ex[i] = fx_mantissa<true>(a[i], &m[i], &bad) + K.e[b][i] + 64;
+    for (int d = 0; d < nt; d++) ex[FX_NB + d] = fx_mantissa<false>(tau[d], &m[FX_NB + d], &bad) + K.e[b][FX_NB] + 64;
+    uint64_t mc;
+    const int ec = fx_mantissa<true>(c0, &mc, &bad) + 64;
+    for (int i = 0; i < FX_NB + nt; i++) E = ex[i] > E ? ex[i] : E;
+    E = ec > E ? ec : E;
+    for (int i = 0; i < FX_NB; i++) o.a[i] = fx_split(fx_scaled(m[i], fx_shift(E, ex[i]), a[i]));
+    for (int d = 0; d < nt; d++) o.t[d] = fx_split(fx_scaled(m[FX_NB + d], fx_shift(E, ex[FX_NB + d]), tau[d]));
+    o.c0 = fx_scaled(mc, fx_shift(E, ec) + 1, c0);
+    o.sh = fx_lift(E);
+}
 
 // One term's products: hi += a.h b.h, cr += a.h b.l + a.l b.h (the low product,
-// below the unit, is dropped). |a.h| <= 2^28, |b.h| <= 2^29: the nine terms of a
-// phase stay below 2^62 in either sum.
+// within 1/4 of the unit either way, is dropped). |a.h| <= 2^30, |b.h| <= 2^29 and
+// |l| <= 2^29: the nine terms of a phase stay below 2^63 in either sum.
 DFI void fx_mac(int64_t &hi, int64_t &cr, fx2 a, fx2 b) {
     hi += (int64_t)a.h * b.h;
     cr += (int64_t)a.h * b.l;

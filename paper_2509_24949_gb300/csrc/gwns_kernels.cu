@@ -270,13 +270,14 @@ __global__ void k_build_fx(Model M, Tables T, const double2 *w64, FxTables X) {
     }
     const int N = M.N;
     for (int j = i0; j < N; j += st) {
+        const int *ex = T.fxk.e[fx_block(T.fxk, j)];
 #pragma unroll
         for (int m = 0; m < NB; m += 2) {
-            const fx2 a = fx_table(T.basis64[(size_t)m * N + j], T.fxe[m]);
-            const fx2 b = fx_table(T.basis64[(size_t)(m + 1) * N + j], T.fxe[m + 1]);
+            const fx2 a = fx_table(T.basis64[(size_t)m * N + j], ex[m]);
+            const fx2 b = fx_table(T.basis64[(size_t)(m + 1) * N + j], ex[m + 1]);
             X.b[(size_t)(m >> 1) * X.n + j] = make_int4(a.h, a.l, b.h, b.l);
         }
-        const fx2 f = fx_table(T.f64[j], T.fxe[NB]);
+        const fx2 f = fx_table(T.f64[j], ex[NB]);
         X.f[j] = make_int2(f.h, f.l);
 #pragma unroll
         for (int d = 0; d < MAXDET; d++) {
@@ -331,15 +332,16 @@ __global__ void k_fx_nodes(Model M, Tables T, const double2 *w64, FxTables X, in
     if (lev == 0) {
         for (int i = threadIdx.x; i < 2 * FX_NODES; i += blockDim.x) {
             const int j = s + i;
-            int64_t hi = X.ref.c0, cr = 0;
+            const FxCoef &q = X.ref[fx_block(T.fxk, j)];
+            int64_t hi = q.c0, cr = FX_HALF;
             for (int m = 0; m < NB; m += 2) {
                 const int4 b = X.b[(size_t)(m >> 1) * X.n + j];
-                fx_mac(hi, cr, X.ref.a[m], fx2{b.x, b.y});
-                fx_mac(hi, cr, X.ref.a[m + 1], fx2{b.z, b.w});
+                fx_mac(hi, cr, q.a[m], fx2{b.x, b.y});
+                fx_mac(hi, cr, q.a[m + 1], fx2{b.z, b.w});
             }
             const int2 f = X.f[j];
-            fx_mac(hi, cr, X.ref.t[0], fx2{f.x, f.y});
-            const fxe E = fx_cis(fx_phase(hi, cr, X.ref.sh), X.sc);
+            fx_mac(hi, cr, q.t[0], fx2{f.x, f.y});
+            const fxe E = fx_cis(fx_phase(hi, cr, q.sh), X.sc);
             const double er = (double)E.rh + (double)E.rl, ei = (double)E.ih + (double)E.il;
             for (int d = 0; d < nd; d++) {
                 const double2 w = w64[(size_t)d * M.N + j];
@@ -357,18 +359,22 @@ __global__ void k_fx_nodes(Model M, Tables T, const double2 *w64, FxTables X, in
         const double f = fma(x, M.df, M.f0);
         double B[NB];
         basis_at(f, B);
-        int64_t hi = X.ref.c0, cr = 0;
+        // in the block of the tile's first bin (fx_layout)
+        const int blk = fx_block(T.fxk, s);
+        const int *ex = T.fxk.e[blk];
+        const FxCoef &q = X.ref[blk];
+        int64_t hi = q.c0, cr = FX_HALF;
 #pragma unroll
         for (int m = 0; m < NB; m += 2) {
-            const fx2 a = fx_table(B[m], T.fxe[m]), b = fx_table(B[m + 1], T.fxe[m + 1]);
+            const fx2 a = fx_table(B[m], ex[m]), b = fx_table(B[m + 1], ex[m + 1]);
             X.b[(size_t)(m >> 1) * X.n + row0 + n] = make_int4(a.h, a.l, b.h, b.l);
-            fx_mac(hi, cr, X.ref.a[m], a);
-            fx_mac(hi, cr, X.ref.a[m + 1], b);
+            fx_mac(hi, cr, q.a[m], a);
+            fx_mac(hi, cr, q.a[m + 1], b);
         }
-        const fx2 ff = fx_table(f, T.fxe[NB]);
+        const fx2 ff = fx_table(f, ex[NB]);
         X.f[row0 + n] = make_int2(ff.h, ff.l);
-        fx_mac(hi, cr, X.ref.t[0], ff);
-        const fxe E = fx_cis(fx_phase(hi, cr, X.ref.sh), X.sc);
+        fx_mac(hi, cr, q.t[0], ff);
+        const fxe E = fx_cis(fx_phase(hi, cr, q.sh), X.sc);
         back[n] = make_double2((double)E.rh + (double)E.rl, -((double)E.ih + (double)E.il));
     }
     __syncthreads();
@@ -1062,12 +1068,13 @@ __global__ void __launch_bounds__(1024) k_rb_fx(int nd, Tables T, RBTables R, RB
         }
     }
     for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+        const int *ex = T.fxk.e[fx_block(T.fxk, e)];
         for (int m = 0; m < NB; m += 2) {
-            const fx2 a = fx_table(R.basis64[(size_t)m * ne + e], T.fxe[m]);
-            const fx2 b = fx_table(R.basis64[(size_t)(m + 1) * ne + e], T.fxe[m + 1]);
+            const fx2 a = fx_table(R.basis64[(size_t)m * ne + e], ex[m]);
+            const fx2 b = fx_table(R.basis64[(size_t)(m + 1) * ne + e], ex[m + 1]);
             X.b[(size_t)(m >> 1) * ne + e] = make_int4(a.h, a.l, b.h, b.l);
         }
-        const fx2 f = fx_table(R.fe[e], T.fxe[NB]);
+        const fx2 f = fx_table(R.fe[e], ex[NB]);
         X.f[e] = make_int2(f.h, f.l);
     }
 }

@@ -107,7 +107,7 @@ struct FxTables {
     // tiles: the reference point, the interpolation matrices [position][node] of a
     // shortest tile's bins and of a tile's two halves' nodes, and two levels'
     // node weights in FP64 (scratch of the build)
-    FxPoint ref;
+    FxCoef ref[FX_BLK];
     double *lag0, *lag1;
     double2 *v[2];
 };
@@ -158,7 +158,7 @@ int ws_blocks_per_sm(int precision, int ndet);
 cudaError_t launch_build_tables(const Model &M, const double *data_re, const double *data_im,
                                 const double *psd, double *basis64, double *f64, double2 *w64,
                                 double *prefix, const MixedTables &X, cudaStream_t s);
-// The FP64 form's split tables from the grid's basis64, f64 and w64 (exponents: Tables::fxe).
+// The FP64 form's split tables from the grid's basis64, f64 and w64 (blocks: Tables::fxk).
 // The cosine and sine table (Tables::fxsc).
 cudaError_t launch_fx_sc(float4 *sc, cudaStream_t s);
 // Relative binning, FP64 form: the split tables from the summary data (RBTables, writable here).

@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(W * 32, EVAL_BLOCKS(PREC, NDET, W)) k_eval(Mod
         if (M.rb) {
             // relative-binning sums: one warp
             if (warp == 0) {
-                const double v = PREC == 0 ? rb_loglike_fx<NDET>(M, T.rb, coef[p], fx, sc)
+                const double v = PREC == 0 ? rb_loglike_fx<NDET>(M, T, coef[p], fx, sc)
                                            : rb_loglike_mixed<NDET>(M, T.rb, coef[p], cm[p], lane);
                 if (lane == 0) {
                     logl[i0 + p] = v;
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(EVAL_FX_W * 32, 16 / EVAL_FX_W) k_eval_fx(Mode
     __syncthreads();
     if constexpr (RB) {
         for (int p = warp; p < np; p += EVAL_FX_W) {
-            const double v = rb_loglike_fx<NDET>(M, T.rb, coef[p], fx[p], sc);
+            const double v = rb_loglike_fx<NDET>(M, T, coef[p], fx[p], sc);
             if (lane == 0) logl[i0 + p] = v;
         }
         if (st && threadIdx.x == 0) atomicAdd(&st->eval_points, (unsigned long long)np);
@@ -1111,7 +1111,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                 __syncwarp();
                 v = rb_loglike_mixed<NDET>(M, T.rb, coef[warp], cm[warp], lane);
             } else {
-                v = rb_loglike_fx<NDET>(M, T.rb, coef[warp], fx[warp], sct);
+                v = rb_loglike_fx<NDET>(M, T, coef[warp], fx[warp], sct);
             }
             if (lane == 0) {
                 lval[warp] = v;
