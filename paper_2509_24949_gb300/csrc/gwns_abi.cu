@@ -334,6 +334,45 @@ int ensure_dead_capacity(ns_ctx *c, long long need) {
     if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; c->graph_k = -1; }
     return NS_OK;
 }
+
+// Mixed form: the tiled form when the Taylor remainder of the basis about each
+// tile's centre stays below 1e-8 rad for every point of the prior, else the
+// per-bin form. The bound: the basis terms of the phase sum to at most twice
+// the Newtonian phase 3/128 (pi T_sun Mc f)^(-5/3) at the lowest chirp mass and
+// frequency (leading-order and 1.5PN terms dominate at f0); the degree-TK
+// remainder of f^(-5/3) over half a tile h is below 4.8 (h/f0)^(TK+1) times the
+// term (TK = 7); a factor 64 covers both with margin. The longest tile that
+// passes, up to 128 bins, is taken: it amortises the per-tile anchor best
+// (GB300, 519,169 bins: degree 6 on 64-bin tiles against degree 7 on 128-bin
+// tiles, batched likelihood 1.53 -> 1.59 M evals/s, slice update 326 -> 304 ms).
+void choose_tiles(Model &M) {
+    M.tlg = 0;
+    M.np = M.N;
+    const double mc = M.lo[P_MC] > 0.0 ? M.lo[P_MC] : 1.0;
+    const double phin = 3.0 / 128.0 * std::pow(M_PI * TSUN * mc * M.f0, -5.0 / 3.0);
+    for (int lg = 7; lg >= 3; lg--) {
+        const double h = 0.5 * (double)(1 << lg) * M.df;
+        if (64.0 * phin * std::pow(h / M.f0, TK + 1) <= 1e-8) {
+            M.tlg = lg;
+            const int gb = 32 << lg;
+            M.np = (M.N + gb - 1) / gb * gb;
+            return;
+        }
+    }
+}
+
+// As alloc_mixed: a tile's anchor values, derivatives and centre, and the padded
+// grid's weights; per bin the basis, f and the weights in float pairs.
+size_t mixed_table_bytes(int N, int n_det, double f0, double df, double mc_lo) {
+    Model M;
+    M.N = N;
+    M.f0 = f0;
+    M.df = df;
+    M.lo[P_MC] = mc_lo;
+    choose_tiles(M);
+    if (!M.tlg) return (size_t)N * (8 * NB + 8 + 8 * n_det);
+    return (size_t)(M.np >> M.tlg) * (16 * NB + 4 * (TK - 1) * NB + 8) + (size_t)M.np * 8 * n_det;
+}
 }  // namespace gwns_host
 
 extern "C" {
@@ -443,32 +482,6 @@ static bool use_df_coefficients(const ns_ctx *c) {
         if (std::fabs(M.lo[p]) > 100.0 || std::fabs(M.hi[p]) > 100.0) return false;
     const char *f = std::getenv("GWNS_COEF_FP64");
     return !(f && f[0] == '1');
-}
-
-// Mixed form: the tiled form when the Taylor remainder of the basis about each
-// tile's centre stays below 1e-8 rad for every point of the prior, else the
-// per-bin form. The bound: the basis terms of the phase sum to at most twice
-// the Newtonian phase 3/128 (pi T_sun Mc f)^(-5/3) at the lowest chirp mass and
-// frequency (leading-order and 1.5PN terms dominate at f0); the degree-TK
-// remainder of f^(-5/3) over half a tile h is below 4.8 (h/f0)^(TK+1) times the
-// term (TK = 7); a factor 64 covers both with margin. The longest tile that
-// passes, up to 128 bins, is taken: it amortises the per-tile anchor best
-// (GB300, 519,169 bins: degree 6 on 64-bin tiles against degree 7 on 128-bin
-// tiles, batched likelihood 1.53 -> 1.59 M evals/s, slice update 326 -> 304 ms).
-static void choose_tiles(Model &M) {
-    M.tlg = 0;
-    M.np = M.N;
-    const double mc = M.lo[P_MC] > 0.0 ? M.lo[P_MC] : 1.0;
-    const double phin = 3.0 / 128.0 * std::pow(M_PI * TSUN * mc * M.f0, -5.0 / 3.0);
-    for (int lg = 7; lg >= 3; lg--) {
-        const double h = 0.5 * (double)(1 << lg) * M.df;
-        if (64.0 * phin * std::pow(h / M.f0, TK + 1) <= 1e-8) {
-            M.tlg = lg;
-            const int gb = 32 << lg;
-            M.np = (M.N + gb - 1) / gb * gb;
-            return;
-        }
-    }
 }
 
 // The same bound at a tile group's lowest frequency f_g, where the phase and

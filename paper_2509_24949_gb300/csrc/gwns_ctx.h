@@ -82,4 +82,6 @@ int choose_slots(const ns_ctx *c);
 int slots_alloc(const ns_ctx *c);
 StepArgs step_args(ns_ctx *c, int k);
 int ensure_dead_capacity(ns_ctx *c, long long need);
+// device bytes of the mixed form's tables of a grid (chirp masses from mc_lo up)
+size_t mixed_table_bytes(int N, int n_det, double f0, double df, double mc_lo);
 }  // namespace gwns_host

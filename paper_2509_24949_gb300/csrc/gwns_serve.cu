@@ -54,15 +54,23 @@ int sampled_dim(const Request &r) {
     return d;
 }
 
-// Device bytes of an analysis apart from its dead list: FP64 basis, f,
-// weighted data, prefix, data and PSD copies; the mixed form's tiled
-// increments, weighted data and tile anchors (grid padded by less than 1024
-// bins); live and final sets; relative-binning tables; fixed overhead.
-size_t footprint_base(const Request &r) {
+// Device bytes of an analysis apart from its dead list, not below what ns_init
+// allocates: FP64 basis, f, data, PSD and prefix; the mixed form's tables (made in
+// both precisions); the FP64 form's weighted data and split tables,
+// with, where node tiles may be chosen (choose_tiles_fx), up to as many node rows
+// as bins (a row per two bins at the shortest tiles, half as many at each next
+// length) and two levels' node weights; live and final sets; relative-binning
+// tables and, while they are built, the fiducial waveform; fixed overhead.
+size_t footprint_base(const Request &r, int precision) {
     const size_t N = r.N, D = r.n_det, n = r.opts.n_live, d = sampled_dim(r);
-    size_t b = (72 + 48 * D) * N + (37 + 8 * D) * (N + 1024);
+    const bool fp64 = precision == NS_FP64;
+    size_t b = (72 + 32 * D) * N + mixed_table_bytes(r.N, r.n_det, r.f0, r.df, r.prior.lo[NS_MC]);
+    if (fp64 && r.coarse_bins == 0) {
+        const bool tiles = N >= 4096 && r.f0 >= 1.0;
+        b += 16 * D * N + (72 + 16 * D) * (tiles ? 2 * N : N) + (tiles ? 12 * D * N : 0);
+    }
     b += n * (16 * d + 40);
-    if (r.coarse_bins > 0) b += (size_t)(r.coarse_bins + 1) * (160 + 64 * D) + 16 * D * N;
+    if (r.coarse_bins > 0) b += (size_t)(r.coarse_bins + 1) * (168 + 72 * D + (fp64 ? 72 + 40 * D : 0)) + 16 * D * N;
     return b + (1u << 20);
 }
 
@@ -72,7 +80,9 @@ size_t dead_bytes(const Request &r, long long cap) { return (size_t)cap * (size_
 // Estimated device bytes at admission: the dead list starts at 64 n entries
 // and doubles when the run outgrows it; the server then adds the growth to the
 // analysis' footprint and to the memory in use (see iterate_all).
-size_t footprint(const Request &r) { return footprint_base(r) + dead_bytes(r, 64LL * r.opts.n_live); }
+size_t footprint(const Request &r, int precision) {
+    return footprint_base(r, precision) + dead_bytes(r, 64LL * r.opts.n_live);
+}
 
 }  // namespace
 
@@ -211,7 +221,7 @@ int iterate_lane(ns_server *s, int L, const std::vector<uint64_t> &ids) {
             // the dead list doubled: count the new size (memory in use is the
             // running analyses' actual footprints, so admission stays within
             // the budget however long the runs grow)
-            const size_t fp = footprint_base(r) + dead_bytes(r, c->dead_cap);
+            const size_t fp = footprint_base(r, s->o.precision) + dead_bytes(r, c->dead_cap);
             if (fp > r.st.footprint) {
                 s->used += fp - r.st.footprint;
                 r.st.footprint = fp;
@@ -389,7 +399,7 @@ int ns_submit(ns_server *s, const ns_request *q, uint64_t *id) {
     std::memset(&r.st, 0, sizeof(r.st));
     r.st.state = NS_REQ_PENDING;
     r.st.t_submit = now(s);
-    r.st.footprint = footprint(r);
+    r.st.footprint = footprint(r, s->o.precision);
     *id = r.id;
     s->reqs.emplace(r.id, std::move(r));
     s->pending.push_back(*id);
