@@ -585,10 +585,10 @@ static int choose_tiles_fx(ns_ctx *c) {
     gwns::FxTiles &X = c->T.tiles;
     if (M.N < 4096 || M.f0 < 1.0) return NS_OK;
     constexpr int m = 1024;
+    std::vector<Coef> cf(m);        // may throw: before the device buffer is taken
     Coef *dev = nullptr;
     int rc = dalloc(&dev, m);
     if (rc) return rc;
-    std::vector<Coef> cf(m);
     cudaError_t e = gwns::launch_prior_coefs(M, c->T, m, dev, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(cf.data(), dev, m * sizeof(Coef), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
