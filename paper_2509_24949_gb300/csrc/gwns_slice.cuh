@@ -139,7 +139,16 @@ constexpr int EVAL_PPC = 4;
 // faster on every grid in tiles of 32 bins or more. GB300, 100 / 8192 draws, before ->
 // now: 3 detectors, 104,000 bins 656 / 1633 -> 478 / 1558 us, 519,169 bins 232 / 4056 ->
 // 200 / 3991; 2 detectors, 31,489 bins 250 / 604 -> 162 / 500; 1 detector, 129,793
-// bins 487 / 1256 -> 387 / 1147.
+// bins 487 / 1256 -> 387 / 1147. The kernels' other calls, left alone -> so, 8192 draws,
+// 3 detectors: shorter tiles (16,225 / 32,449 bins) 97 / 132 -> 78 / 99 us, bin by bin
+// (4017) 74 -> 62, physical parameters (4017 / 32,449 bins) 326 / 718 -> 207 / 406,
+// relative binning 525 -> 327; 64 draws of any of them lose up to 2 us. One detector in
+// CTAs of 4 warps: 5 of them, 4017 bins 8192 draws 55.7 us (4: 58.5, 6: 56.9, left alone
+// 61.2). Four detectors' tile loop on tiles of 32 bins or
+// more wants 3 CTAs of 4 warps (EVAL_BATCH4_BLOCKS): at 4 its registers spill, 32 s
+// (64,897 bins) 64 / 8192 draws 56 / 121 -> 49 / 118 us, 64 s of low masses 720 / 2124 ->
+// 486 / 1927; on shorter tiles 4 stay better (4017 bins, 8192 draws 71 -> 66).
+#define EVAL_BATCH4_BLOCKS 3
 #define EVAL_BATCH_BLOCKS(NDET, W) ((NDET) == 1 ? ((W) == 4 ? 5 : 32 / (W)) : 16 / (W))
 #define EVAL_BLOCKS(PREC, NDET, W) ((PREC) == 0 ? 16 / (W) : (NDET) == 1 ? 32 / (W) : (NDET) == 2 ? 20 / (W) : 16 / (W))
 
@@ -216,9 +225,9 @@ __global__ void __launch_bounds__(W * 32, EVAL_BLOCKS(PREC, NDET, W)) k_eval(Mod
 // 8192 prior draws of the 64,897-bin workload: the previous kernel (coefficients
 // of four points on one warp, the other warp waiting, every point's tile groups
 // shared by both warps and reduced in FP64) reached 5.75e7 evals/s.
-template <int NDET, int W>
-__global__ void __launch_bounds__(W * 32, EVAL_BATCH_BLOCKS(NDET, W)) k_eval_batch(Model M, Tables T, const double *in, int m, double *logl,
-                                                       RunState *st) {
+template <int NDET, int W, int BLOCKS = EVAL_BATCH_BLOCKS(NDET, W)>
+__global__ void __launch_bounds__(W * 32, BLOCKS) k_eval_batch(Model M, Tables T, const double *in, int m, double *logl,
+                                                               RunState *st) {
     constexpr int NG = W >= 2 ? W / 2 : 1;
     constexpr int PPC = 4 * NG;
     __shared__ Coef coef[PPC];
@@ -360,7 +369,13 @@ cudaError_t eval_launch(const Model &M, const Tables &T, int warps, const double
             switch (warps) {
                 case 1: k_eval_batch<NDET, 1><<<gb, 32, 0, s>>>(M, T, in, m, logl, st); break;
                 case 2: k_eval_batch<NDET, 2><<<gb, 64, 0, s>>>(M, T, in, m, logl, st); break;
-                case 4: k_eval_batch<NDET, 4><<<gb, 128, 0, s>>>(M, T, in, m, logl, st); break;
+                case 4:
+                    if (NDET == 4 && M.tlg >= 5)
+                        k_eval_batch<NDET, 4, NDET == 4 ? EVAL_BATCH4_BLOCKS : EVAL_BATCH_BLOCKS(NDET, 4)>
+                            <<<gb, 128, 0, s>>>(M, T, in, m, logl, st);
+                    else
+                        k_eval_batch<NDET, 4><<<gb, 128, 0, s>>>(M, T, in, m, logl, st);
+                    break;
                 default: k_eval_batch<NDET, 8><<<gb, 256, 0, s>>>(M, T, in, m, logl, st); break;
             }
             return cudaGetLastError();
