@@ -220,7 +220,7 @@ int build_rb(ns_ctx *c) {
 }
 
 int eval_points(ns_ctx *c, const double *in, int is_theta, int m, double *logl) {
-    CK(launch_eval(c->M, c->T, c->precision, choose_warps(c), in, is_theta, m, logl, c->state, c->stream));
+    CK(launch_eval(c->M, c->T, c->precision, choose_warps(c), c->n_sm, in, is_theta, m, logl, c->state, c->stream));
     return NS_OK;
 }
 
@@ -245,9 +245,9 @@ int choose_slots(const ns_ctx *c) {
     }
     if (c->M.model == M_TOY) return 1;
     const int bins = c->M.rb ? c->T.rb.nb : c->M.N;
-    // measured on GB300 (512 / 4017 / 64,897-bin workloads): FP64 binds on its
-    // pipe beyond small grids (one slot plus tail speculation from 64,897 bins),
-    // the mixed form on latency up to large grids
+    // measured on GB300 (512 / 4017 / 64,897-bin workloads; the FP64 counts while its
+    // bins still ran on the FP64 pipe, which bound beyond small grids: one slot plus
+    // tail speculation from 64,897 bins); the mixed form waits for latency up to large grids
     if (c->precision == NS_FP64) return bins <= 1024 ? 4 : (bins <= 16384 ? 2 : 1);
     return bins <= 1024 ? 8 : (c->M.coop ? 2 : 4);
 }
@@ -1223,10 +1223,10 @@ int ns_autotune_eval(ns_ctx *c, int trials, int *warps) {
     cudaError_t e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     for (int i = 0; i < 4 && e == cudaSuccess; i++) {
-        e = launch_eval(c->M, c->T, c->precision, cand[i], c->live_u, 0, m, out, nullptr, c->stream);
+        e = launch_eval(c->M, c->T, c->precision, cand[i], c->n_sm, c->live_u, 0, m, out, nullptr, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
         for (int t = 0; t < trials && e == cudaSuccess; t++)
-            e = launch_eval(c->M, c->T, c->precision, cand[i], c->live_u, 0, m, out, nullptr, c->stream);
+            e = launch_eval(c->M, c->T, c->precision, cand[i], c->n_sm, c->live_u, 0, m, out, nullptr, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.f;

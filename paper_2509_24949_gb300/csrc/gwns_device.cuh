@@ -1356,42 +1356,30 @@ __device__ __forceinline__ void tile_pairs(const float4 *w4, size_t dstride, int
 }
 
 // Short tiles (L <= 16): every detector's phase reduced mod 1 and its own
-// FP32 __sincosf per bin, the nc <= NC candidates sharing the table loads (on
-// few bins per tile the rotation's per-tile setup and the candidates taken one
-// after the other cost more than the sines save). Same sums as tile_bins.
-template <int NDET, int NC>
-__device__ __forceinline__ void tile_bins_direct(const Tables &T, int lg, int np, const CoefMixed *cm,
-                                          const int *jcut, int nc, int g0, int gstride,
-                                          float zh[NC][NDET][2], float zl[NC][NDET][2],
-                                          int g_end = 0x7fffffff) {
+// FP32 __sincosf per bin (on few bins per tile the rotation's per-tile setup costs
+// more than the sines save). Same sums as tile_bins.
+template <int NDET>
+__device__ __forceinline__ void tile_bins_direct(const Tables &T, int lg, int np, const CoefMixed &cm, const int &jcut,
+                                                 int g0, int gstride, float (&zh)[NDET][2], float (&zl)[NDET][2],
+                                                 int g_end = 0x7fffffff) {
     const int lane = threadIdx.x & 31;
     const int L = 1 << lg, half = L >> 1, nt = np >> lg;
 #pragma unroll
-    for (int c = 0; c < NC; c++)
-#pragma unroll
-        for (int d = 0; d < NDET; d++) zh[c][d][0] = zh[c][d][1] = zl[c][d][0] = zl[c][d][1] = 0.f;
-    int jmax = -1;
-#pragma unroll
-    for (int c = 0; c < NC; c++)
-        if (c < nc) jmax = max(jmax, jcut[c]);
-    const int ngroups = min(jmax < 0 ? 0 : (jmax >> (lg + 5)) + 1, g_end);
+    for (int d = 0; d < NDET; d++) zh[d][0] = zh[d][1] = zl[d][0] = zl[d][1] = 0.f;
+    const int ngroups = min(jcut < 0 ? 0 : (jcut >> (lg + 5)) + 1, g_end);
     const float4 *wt4 = reinterpret_cast<const float4 *>(T.wt);
     for (int g = g0; g < ngroups; g += gstride) {
         const int t = (g << 5) + lane, s = t << lg;
-        int cnt[NC];
-        int nmax = 0;
-        float c1h[NC], c1l[NC], ck[NC][TK - 1], Ah[NC][NDET], Al[NC][NDET];
+        const int cnt = min(max(jcut - s + 1, 0), L), nmax = min(max(jcut - (g << (lg + 5)) + 1, 0), L);
+        float c1h, c1l, ck[TK - 1], Ah[NDET], Al[NDET];
         const float2 fc = __ldg(T.fc + t);
+        {
+            float sh = cm.c0h, sl = cm.c0l, h1 = 0.f, l1 = 0.f;
 #pragma unroll
-        for (int c = 0; c < NC; c++) {
-            cnt[c] = (c < nc) ? min(max(jcut[c] - s + 1, 0), L) : 0;
-            nmax = max(nmax, (c < nc) ? min(max(jcut[c] - (g << (lg + 5)) + 1, 0), L) : 0);
-            float sh = cm[c].c0h, sl = cm[c].c0l, h1 = 0.f, l1 = 0.f;
-#pragma unroll
-            for (int k = 0; k < TK - 1; k++) ck[c][k] = 0.f;
+            for (int k = 0; k < TK - 1; k++) ck[k] = 0.f;
 #pragma unroll
             for (int m = 0; m < NB; m++) {
-                const float ah = cm[c].ah[m], al = cm[c].al[m];
+                const float ah = cm.ah[m], al = cm.al[m];
                 // anchor term a_m B_m(f_c)
                 const float2 b0 = __ldg(T.tb0 + (size_t)m * nt + t);
                 float p = ah * b0.x;
@@ -1413,29 +1401,27 @@ __device__ __forceinline__ void tile_bins_direct(const Tables &T, int lg, int np
                 l1 += e2 + e;
 #pragma unroll
                 for (int k = 0; k < TK - 1; k++)
-                    ck[c][k] = fmaf(ah, __ldg(T.tbk + ((size_t)k * NB + m) * nt + t), ck[c][k]);
+                    ck[k] = fmaf(ah, __ldg(T.tbk + ((size_t)k * NB + m) * nt + t), ck[k]);
             }
-            c1h[c] = h1 + l1;
-            c1l[c] = l1 - (c1h[c] - h1);
+            c1h = h1 + l1;
+            c1l = l1 - (c1h - h1);
             sh -= rintf(sh);
 #pragma unroll
             for (int d = 0; d < NDET; d++) {
-                const float th = cm[c].tauh[d], tl = cm[c].taul[d];
+                const float th = cm.tauh[d], tl = cm.taul[d];
                 const float p = th * fc.x;
                 float e = fmaf(th, fc.x, -p);
                 e = fmaf(th, fc.y, e);
                 e = fmaf(tl, fc.x, e);
                 float s2, e2;
                 two_sum(sh, p, s2, e2);
-                Ah[c][d] = s2 - rintf(s2);
-                Al[c][d] = sl + (e2 + e);
+                Ah[d] = s2 - rintf(s2);
+                Al[d] = sl + (e2 + e);
             }
         }
-        float pr[NC][NDET], pim[NC][NDET];
+        float pr[NDET], pim[NDET];
 #pragma unroll
-        for (int c = 0; c < NC; c++)
-#pragma unroll
-            for (int d = 0; d < NDET; d++) pr[c][d] = pim[c][d] = 0.f;
+        for (int d = 0; d < NDET; d++) pr[d] = pim[d] = 0.f;
         const size_t gb = (size_t)g << (lg + 5);
         for (int q = 0; q < nmax; q += 4) {
             float4 w[NDET][2];
@@ -1449,38 +1435,34 @@ __device__ __forceinline__ void tile_bins_direct(const Tables &T, int lg, int np
             for (int r = 0; r < 4; r++) {
                 const int i = q + r;
                 const float x = (float)(i - half);
+                if (i < cnt) {
+                    const float p = c1h * x;
+                    const float e = fmaf(c1h, x, -p);
+                    float hq = ck[TK - 2];
 #pragma unroll
-                for (int c = 0; c < NC; c++) {
-                    if (i >= cnt[c]) continue;
-                    const float p = c1h[c] * x;
-                    const float e = fmaf(c1h[c], x, -p);
-                    float hq = ck[c][TK - 2];
-#pragma unroll
-                    for (int k = TK - 3; k >= 0; k--) hq = fmaf(hq, x, ck[c][k]);
-                    hq = fmaf(hq, x, c1l[c]);
+                    for (int k = TK - 3; k >= 0; k--) hq = fmaf(hq, x, ck[k]);
+                    hq = fmaf(hq, x, c1l);
                     const float sm = fmaf(hq, x, e);
                     const float P = p - rintf(p);
 #pragma unroll
                     for (int d = 0; d < NDET; d++) {
-                        const float y = (P + Ah[c][d]) + (sm + fmaf(x, cm[c].dtau[d], Al[c][d]));
+                        const float y = (P + Ah[d]) + (sm + fmaf(x, cm.dtau[d], Al[d]));
                         const float red = y - rintf(y);
                         float sv, cv;
                         __sincosf(red * 6.283185307179586f, &sv, &cv);
                         const float4 ww = w[d][r >> 1];
                         const float wr = (r & 1) ? ww.y : ww.x, wi = (r & 1) ? ww.w : ww.z;
-                        pr[c][d] = fmaf(wr, cv, fmaf(-wi, sv, pr[c][d]));
-                        pim[c][d] = fmaf(wr, sv, fmaf(wi, cv, pim[c][d]));
+                        pr[d] = fmaf(wr, cv, fmaf(-wi, sv, pr[d]));
+                        pim[d] = fmaf(wr, sv, fmaf(wi, cv, pim[d]));
                     }
                 }
             }
         }
 #pragma unroll
-        for (int c = 0; c < NC; c++)
-#pragma unroll
-            for (int d = 0; d < NDET; d++) {
-                df_acc(zh[c][d][0], zl[c][d][0], pr[c][d]);
-                df_acc(zh[c][d][1], zl[c][d][1], pim[c][d]);
-            }
+        for (int d = 0; d < NDET; d++) {
+            df_acc(zh[d][0], zl[d][0], pr[d]);
+            df_acc(zh[d][1], zl[d][1], pim[d]);
+        }
     }
 }
 // One candidate over tile group g (its 32 tiles, one per lane) by rotation,
@@ -1557,56 +1539,41 @@ __device__ __forceinline__ void rot_group(const Tables &T, int lg, int np, const
         tile_pairs<NDET, true, PF, K>(w4, dstride, lane, half, (nmax + 7) & ~7, cnt, k, cm, zr, zi);
 }
 
-// One warp's double-float sums over tile groups g0, g0 + gstride, ... for nc <= NC
-// candidates (coefficients cm[c], last bins jcut[c]): zh/zl[c][d][0/1] =
-// real/imaginary part of sum_j w_dj exp(2 pi i phase_dj), not yet reduced over
-// the warp. Detector 0 direct and the others by their rotation, one candidate
-// after the other. With LO, groups g >= T.g_lo take the Taylor degree TK_LO and
-// the rest TK (GB300, 519,169 bins: slice update 205.8 -> 192.3 ms); without it
-// every group takes TK, one copy of the tile code (the c2 slice update, bound by
-// latency and instruction fetch, runs 13.5 ms with one copy and 14.5 with two).
-template <int NDET, int NC, bool PF, bool LO>
-__device__ __forceinline__ void tile_bins_rot(const Tables &T, int lg, int np, const CoefMixed *cm,
-                                              const int *jcut, int nc, int g0, int gstride,
-                                              float zh[NC][NDET][2], float zl[NC][NDET][2],
+// One warp's double-float sums over tile groups g0, g0 + gstride, ... of a
+// candidate (coefficients cm, last bin jcut): zh/zl[d][0/1] = real/imaginary part
+// of sum_j w_dj exp(2 pi i phase_dj), not yet reduced over the warp. Detector 0
+// direct and the others by their rotation. With LO, groups g >= T.g_lo take the
+// Taylor degree TK_LO and the rest TK (GB300, 519,169 bins: slice update 205.8 ->
+// 192.3 ms); without it every group takes TK, one copy of the tile code (the c2
+// slice update, bound by latency and instruction fetch, runs 13.5 ms with one copy
+// and 14.5 with two). jcut by reference, read again from shared memory per group: in a
+// register it makes the three-detector kernels spill (8192 draws on 519,169 bins 3.98 ->
+// 4.05 ms).
+template <int NDET, bool PF, bool LO>
+__device__ __forceinline__ void tile_bins_rot(const Tables &T, int lg, int np, const CoefMixed &cm, const int &jcut,
+                                              int g0, int gstride, float (&zh)[NDET][2], float (&zl)[NDET][2],
                                               int g_end = 0x7fffffff) {
+    float ah[NDET][2], al[NDET][2];
 #pragma unroll
-    for (int c = 0; c < NC; c++)
+    for (int d = 0; d < NDET; d++) ah[d][0] = ah[d][1] = al[d][0] = al[d][1] = 0.f;
+    const int ngroups = min(jcut < 0 ? 0 : (jcut >> (lg + 5)) + 1, g_end);
+    for (int g = g0; g < ngroups; g += gstride) {
+        if (jcut < (g << (lg + 5))) continue;
+        float zr[NDET], zi[NDET];
+        if (LO && g >= T.g_lo)
+            rot_group<NDET, PF, TK_LO>(T, lg, np, cm, jcut, g, zr, zi);
+        else
+            rot_group<NDET, PF, TK>(T, lg, np, cm, jcut, g, zr, zi);
 #pragma unroll
-        for (int d = 0; d < NDET; d++) zh[c][d][0] = zh[c][d][1] = zl[c][d][0] = zl[c][d][1] = 0.f;
-    // candidates one after the other (a run-time loop: one copy of the tile
-    // code, so the kernels' hot code is smaller; GB300: 64,897 bins, slice
-    // update 14.7 -> 13.9 ms; 519,169 bins, 249 -> 244 ms), each over its own
-    // groups in order, so each candidate's sums are the same as with the
-    // candidates taken in turn over each group
-#pragma unroll 1
-    for (int c = 0; c < nc; c++) {
-        float ah[NDET][2], al[NDET][2];
-#pragma unroll
-        for (int d = 0; d < NDET; d++) ah[d][0] = ah[d][1] = al[d][0] = al[d][1] = 0.f;
-        const int ngroups = min(jcut[c] < 0 ? 0 : (jcut[c] >> (lg + 5)) + 1, g_end);
-        for (int g = g0; g < ngroups; g += gstride) {
-            if (jcut[c] < (g << (lg + 5))) continue;
-            float zr[NDET], zi[NDET];
-            if (LO && g >= T.g_lo)
-                rot_group<NDET, PF, TK_LO>(T, lg, np, cm[c], jcut[c], g, zr, zi);
-            else
-                rot_group<NDET, PF, TK>(T, lg, np, cm[c], jcut[c], g, zr, zi);
-#pragma unroll
-            for (int d = 0; d < NDET; d++) {
-                df_acc(ah[d][0], al[d][0], zr[d]);
-                df_acc(ah[d][1], al[d][1], zi[d]);
-            }
+        for (int d = 0; d < NDET; d++) {
+            df_acc(ah[d][0], al[d][0], zr[d]);
+            df_acc(ah[d][1], al[d][1], zi[d]);
         }
+    }
 #pragma unroll
-        for (int cc = 0; cc < NC; cc++)
-            if (cc == c) {
-#pragma unroll
-                for (int d = 0; d < NDET; d++) {
-                    zh[cc][d][0] = ah[d][0]; zh[cc][d][1] = ah[d][1];
-                    zl[cc][d][0] = al[d][0]; zl[cc][d][1] = al[d][1];
-                }
-            }
+    for (int d = 0; d < NDET; d++) {
+        zh[d][0] = ah[d][0]; zh[d][1] = ah[d][1];
+        zl[d][0] = al[d][0]; zl[d][1] = al[d][1];
     }
 }
 // The tiled form's sums, by rotation (ROT: tiles of 32 bins or more; GB300,
@@ -1614,15 +1581,14 @@ __device__ __forceinline__ void tile_bins_rot(const Tables &T, int lg, int np, c
 // 32-bin tiles: 14.3 -> 13.8 ms) or direct (shorter tiles, where the per-tile
 // rotation setup outweighs the saved sines: 64,897 bins in 16-bin tiles, 14.3
 // against 15.9 ms by rotation). Callers choose by the tile length.
-template <int NDET, int NC, bool ROT, bool PF = false, bool LO = false>
-__device__ __forceinline__ void tile_bins(const Tables &T, int lg, int np, const CoefMixed *cm,
-                                          const int *jcut, int nc, int g0, int gstride,
-                                          float zh[NC][NDET][2], float zl[NC][NDET][2],
+template <int NDET, bool ROT, bool PF = false, bool LO = false>
+__device__ __forceinline__ void tile_bins(const Tables &T, int lg, int np, const CoefMixed &cm, const int &jcut, int g0,
+                                          int gstride, float (&zh)[NDET][2], float (&zl)[NDET][2],
                                           int g_end = 0x7fffffff) {
     if constexpr (ROT)
-        tile_bins_rot<NDET, NC, PF, LO>(T, lg, np, cm, jcut, nc, g0, gstride, zh, zl, g_end);
+        tile_bins_rot<NDET, PF, LO>(T, lg, np, cm, jcut, g0, gstride, zh, zl, g_end);
     else
-        tile_bins_direct<NDET, NC>(T, lg, np, cm, jcut, nc, g0, gstride, zh, zl, g_end);
+        tile_bins_direct<NDET>(T, lg, np, cm, jcut, g0, gstride, zh, zl, g_end);
 }
 
 // Double-float warp sum (TwoSum of the high parts, low parts added).
@@ -1688,7 +1654,7 @@ __device__ __forceinline__ void warp_sum_df_many(float (&h)[16], float (&l)[16],
 // edge G is its lower bin's part alone (GR). One warp, 31 bins a pass, in the
 // split arithmetic of gwns_fx.cuh: about 600 cycles a pass and three detectors,
 // against 11,000 for the FP64 sines, cosines and sums. GB300, 8192 draws on 1024
-// coarse bins: 2.81 ms -> 237 us.
+// coarse bins: 2.81 ms -> 245 us.
 template <int NDET>
 __device__ __forceinline__ double rb_loglike_fx(const Model &M, const Tables &T, const Coef &c, const FxPoint &fx,
                                                 const float4 *sc) {

@@ -143,7 +143,7 @@ cudaError_t noalloc_scratch_address(double **ptr);
 // Likelihood and slice-update launchers per (precision, detectors), defined in
 // gwns_slice.cuh and instantiated in gwns_inst_p<P>_d<D>.cu.
 template <int PREC, int NDET>
-cudaError_t eval_launch(const Model &M, const Tables &T, int warps, const double *in, int th, int m,
+cudaError_t eval_launch(const Model &M, const Tables &T, int warps, int n_sm, const double *in, int th, int m,
                         double *logl, RunState *st, cudaStream_t s);
 template <int PREC, int NDET>
 cudaError_t slice_launch(const Model &M, const Tables &T, int slots, const StepArgs &A, cudaStream_t s);
@@ -174,7 +174,7 @@ cudaError_t launch_rb_fx(const Model &M, const Tables &T, const RBTables &R, con
 cudaError_t launch_prior_coefs(const Model &M, const Tables &T, int m, Coef *out, cudaStream_t s);
 cudaError_t launch_build_fx(const Model &M, const Tables &T, const double2 *w64, const FxTables &X, cudaStream_t s);
 cudaError_t launch_init_live(const Model &M, uint64_t seed, int n, double *live_u, cudaStream_t s);
-cudaError_t launch_eval(const Model &M, const Tables &T, int precision, int warps, const double *in,
+cudaError_t launch_eval(const Model &M, const Tables &T, int precision, int warps, int n_sm, const double *in,
                         int in_is_theta, int m, double *logl, RunState *st, cudaStream_t s);
 cudaError_t launch_select(const double *logl, int n, int *order, cudaStream_t s);
 cudaError_t launch_evidence(const Model &M, const StepArgs &A, cudaStream_t s);

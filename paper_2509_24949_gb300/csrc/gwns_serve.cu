@@ -208,7 +208,8 @@ int iterate_lane(ns_server *s, int L, const std::vector<uint64_t> &ids) {
     // analysis always runs at its own width, whatever the mix. Tiled mixed grids
     // take the direct form at every tile length (GB300, the 64-analysis stream:
     // p50 / p99 4.55 / 7.7 s; with the rotation form for tiles of 32 bins or more
-    // in a kernel of its own, 5.8 / 9.2 s, and 6.3 / 10.0 s on a second stream)
+    // in a kernel of its own, 5.8 / 9.2 s, and 6.3 / 10.0 s on a second stream;
+    // measured while the direct form shared a table load between two candidates)
     std::map<std::pair<int, int>, std::vector<int2>> groups;
     for (int a = 0; a < na; a++) {
         Request &r = s->reqs[ids[a]];

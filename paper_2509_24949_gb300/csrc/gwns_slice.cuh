@@ -73,12 +73,12 @@ __device__ __forceinline__ void cta_loglike_bins(const Model &M, const Tables &T
         warp_sums_df_to<NDET>(zh, zl, red[warp], T.fxs);
     } else if (M.tlg) {
         // tiled form: warp w takes tile groups w, w + W, ...
-        float zh[1][NDET][2], zl[1][NDET][2];
+        float zh[NDET][2], zl[NDET][2];
         if (M.tlg >= 5)
-            tile_bins<NDET, 1, true, true, true>(T, M.tlg, M.np, &cm, &coef.jcut, 1, warp, W, zh, zl);
+            tile_bins<NDET, true, true, true>(T, M.tlg, M.np, cm, coef.jcut, warp, W, zh, zl);
         else
-            tile_bins<NDET, 1, false>(T, M.tlg, M.np, &cm, &coef.jcut, 1, warp, W, zh, zl);
-        warp_sums_df_to<NDET>(zh[0], zl[0], red[warp]);
+            tile_bins<NDET, false>(T, M.tlg, M.np, cm, coef.jcut, warp, W, zh, zl);
+        warp_sums_df_to<NDET>(zh, zl, red[warp]);
     } else {
         float zh[NDET][2], zl[NDET][2];
         bins_mixed<NDET>(T, M.N, cm, coef.jcut, threadIdx.x, W * 32, zh, zl);
@@ -263,12 +263,12 @@ __global__ void __launch_bounds__(W * 32, BLOCKS) k_eval_batch(Model M, Tables T
     for (int p = warp; p < np; p += W) {
         double t;       // on lane 0: sum over detectors of Re(G_d Z_d)
         if (M.tlg) {
-            float zh[1][NDET][2], zl[1][NDET][2];
+            float zh[NDET][2], zl[NDET][2];
             if (M.tlg >= 5)
-                tile_bins<NDET, 1, true, true>(T, M.tlg, M.np, &cm[p], &coef[p].jcut, 1, 0, 1, zh, zl);
+                tile_bins<NDET, true, true>(T, M.tlg, M.np, cm[p], coef[p].jcut, 0, 1, zh, zl);
             else
-                tile_bins<NDET, 1, false>(T, M.tlg, M.np, &cm[p], &coef[p].jcut, 1, 0, 1, zh, zl);
-            t = warp_detector_terms_df<NDET>(zh[0], zl[0], coef[p]);
+                tile_bins<NDET, false>(T, M.tlg, M.np, cm[p], coef[p].jcut, 0, 1, zh, zl);
+            t = warp_detector_terms_df<NDET>(zh, zl, coef[p]);
         } else {
             float zh[NDET][2], zl[NDET][2];
             bins_mixed<NDET>(T, M.N, cm[p], coef[p].jcut, lane, 32, zh, zl);
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(EVAL_FX_W * 32, 16 / EVAL_FX_W) k_eval_fx(Mode
 }
 
 template <int PREC, int NDET>
-cudaError_t eval_launch(const Model &M, const Tables &T, int warps, const double *in, int th, int m,
+cudaError_t eval_launch(const Model &M, const Tables &T, int warps, int n_sm, const double *in, int th, int m,
                         double *logl, RunState *st, cudaStream_t s) {
     const int nbins = M.rb ? T.rb.nb : M.N;
     if constexpr (PREC == 1) {
@@ -385,7 +385,7 @@ cudaError_t eval_launch(const Model &M, const Tables &T, int warps, const double
         if (M.model == M_GW && !th) {
             // as many points a CTA as leave a CTA for every SM
             int P = 1;
-            while (P < EVAL_FX_P && m >= 2 * P * 152) P *= 2;
+            while (P < EVAL_FX_P && m >= 2 * P * n_sm) P *= 2;
             if (M.rb) k_eval_fx<NDET, true><<<(m + P - 1) / P, EVAL_FX_W * 32, 0, s>>>(M, T, in, m, P, 1, logl, st);
             else k_eval_fx<NDET, false><<<(m + P - 1) / P, EVAL_FX_W * 32, 0, s>>>(M, T, in, m, P, warps, logl, st);
             return cudaGetLastError();
@@ -830,16 +830,16 @@ __device__ __forceinline__ void ws_chunk(const Model &M, const Tables &T, const 
     const int lane = threadIdx.x & 31;
     const int g0 = c * G, g1 = g0 + G;
     for (int c0 = 0; c0 < ns; c0++) {
-        float zh[1][NDET][2], zl[1][NDET][2];
-        tile_bins<NDET, 1, true, true, true>(T, M.tlg, M.np, cm + c0, jc + c0, 1, g0, 1, zh, zl, g1);
+        float zh[NDET][2], zl[NDET][2];
+        tile_bins<NDET, true, true, true>(T, M.tlg, M.np, cm[c0], jc[c0], g0, 1, zh, zl, g1);
         // value v = (detector, re/im), summed over the warp at once
         float vh[16], vl[16];
 #pragma unroll
         for (int dd = 0; dd < NDET; dd++)
 #pragma unroll
             for (int ri = 0; ri < 2; ri++) {
-                vh[dd * 2 + ri] = zh[0][dd][ri];
-                vl[dd * 2 + ri] = zl[0][dd][ri];
+                vh[dd * 2 + ri] = zh[dd][ri];
+                vl[dd * 2 + ri] = zl[dd][ri];
             }
         float rh, rl;
         warp_sum_df_many<2 * NDET>(vh, vl, rh, rl);
@@ -986,11 +986,10 @@ __device__ void ws_help(const Model &M, const Tables &T, const StepArgs &A) {
 // all others (shorter tiles, per-bin grids, FP64).
 enum { FORM_DIRECT = 0, FORM_ROT = 2 };
 
-template <int NDET, int NC, int FORM>
-__device__ __forceinline__ void tile_bins_form(const Model &M, const Tables &T, const CoefMixed *cm,
-                                               const int *jc, int nc, int g0, int gstride,
-                                               float zh[NC][NDET][2], float zl[NC][NDET][2]) {
-    tile_bins<NDET, NC, FORM == FORM_ROT>(T, M.tlg, M.np, cm, jc, nc, g0, gstride, zh, zl);
+template <int NDET, int FORM>
+__device__ __forceinline__ void tile_bins_form(const Model &M, const Tables &T, const CoefMixed &cm, const int &jc,
+                                               int g0, int gstride, float (&zh)[NDET][2], float (&zl)[NDET][2]) {
+    tile_bins<NDET, FORM == FORM_ROT>(T, M.tlg, M.np, cm, jc, g0, gstride, zh, zl);
 }
 
 template <int PREC, int NDET, int S, int W, int FORM, bool WS = false>
@@ -1134,8 +1133,7 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
             }
         } else if (PREC == 1 && S > 1 && S <= 4 && M.model == M_GW && !M.rb && M.coop) {
             // mixed, every warp on every candidate of the round: the tiled form
-            // shares out the tile groups (two candidates per pass on one table
-            // load), the per-bin form strides the bins
+            // shares out the tile groups, the per-bin form strides the bins
             if (warp < ns && !M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, FORM == FORM_ROT);
             if (lane == 0 && warp < ns) jc[warp] = coef[warp].jcut;
             __syncthreads();
@@ -1156,9 +1154,9 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                     const int ng = jc[c0] < 0 ? 0 : (jc[c0] >> (M.tlg + 5)) + 1;
                     for (int r = 0; r < min(ng, W); r++, it++) {
                         if ((it & (W - 1)) != warp) continue;
-                        float zh[1][NDET][2], zl[1][NDET][2];
-                        tile_bins_form<NDET, 1, FORM>(M, T, cm + c0, jc + c0, 1, r, W, zh, zl);
-                        warp_sums_df_to<NDET>(zh[0], zl[0], &part[r][c0][0][0]);
+                        float zh[NDET][2], zl[NDET][2];
+                        tile_bins_form<NDET, FORM>(M, T, cm[c0], jc[c0], r, W, zh, zl);
+                        warp_sums_df_to<NDET>(zh, zl, &part[r][c0][0][0]);
                     }
                 }
             } else {
@@ -1192,9 +1190,9 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                 if (dd == 0 && sc < ns && lane < S * NDET) lval[sc] = t - 0.5 * coef[sc].hh;
             }
         } else if (PREC == 0 && W > 1 && M.model == M_GW && !M.rb && tailmode == 2) {
-            // FP64 above 1024 bins: each candidate's bins on two warps (warps on
-            // different SM sub-partitions issue FP64 independently), bin j on
-            // lane j mod 32 of warp (j / 32) mod 2; the two warp sums meet in
+            // FP64 above 1024 bins: each candidate's bins on two warps (on different
+            // SM sub-partitions, each with its own FP32 and integer issue), row r on
+            // lane r mod 32 of warp (r / 32) mod 2; the two warp sums meet in
             // shared memory in a fixed order, whatever the round.
             const int lg = 1;
             const int wpc = 1 << lg, cand = warp >> lg, sub = warp & (wpc - 1);
@@ -1232,9 +1230,9 @@ __device__ void slice_body(const Model &M, const Tables &T, const StepArgs &A, c
                 if (!M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, FORM == FORM_ROT);
                 if (lane == 0) jc[warp] = coef[warp].jcut;
                 __syncwarp();
-                float zh[1][NDET][2], zl[1][NDET][2];
-                tile_bins_form<NDET, 1, FORM>(M, T, &cm[warp], &jc[warp], 1, 0, 1, zh, zl);
-                v = warp_detector_terms_df<NDET>(zh[0], zl[0], coef[warp]);
+                float zh[NDET][2], zl[NDET][2];
+                tile_bins_form<NDET, FORM>(M, T, cm[warp], jc[warp], 0, 1, zh, zl);
+                v = warp_detector_terms_df<NDET>(zh, zl, coef[warp]);
             } else {
                 if (!M.cdf) coef_to_mixed_warp(coef[warp], M.n_det, M.df, &cm[warp], nullptr, FORM == FORM_ROT);
                 __syncwarp();
@@ -1338,18 +1336,12 @@ cudaError_t slice_launch(const Model &M, const Tables &T, int slots, const StepA
     // finish sooner (GB300, 519,169 bins: 536 -> 467 ms per slice update; on
     // 64,897 bins, where an evaluation has a few tile groups, 15.2 -> 17.5 ms,
     // hence the threshold)
-    if (PREC == 1 && slots == 4 && M.model == M_GW && M.coop && M.tlg >= 5 && !M.rb &&
-        M.N >= 262144) {
-        if constexpr (PREC == 1) {
-            if (A.ws) {
-                k_slice_ws<NDET><<<A.ws_nslot, 256, 0, s>>>(M, T, A);
-                return cudaGetLastError();
-            }
-        }
-        k_slice<PREC, NDET, 4, 8, FORM_ROT><<<A.k, 256, 0, s>>>(M, T, A);
-        return cudaGetLastError();
-    }
     if constexpr (PREC == 1) {
+        if (slots == 4 && M.model == M_GW && M.coop && M.tlg >= 5 && !M.rb && M.N >= 262144) {
+            if (A.ws) k_slice_ws<NDET><<<A.ws_nslot, 256, 0, s>>>(M, T, A);
+            else k_slice<PREC, NDET, 4, 8, FORM_ROT><<<A.k, 256, 0, s>>>(M, T, A);
+            return cudaGetLastError();
+        }
         if (M.tlg >= 5) return slice_launch_form<PREC, NDET, FORM_ROT>(M, T, slots, A, s);
     }
     return slice_launch_form<PREC, NDET, FORM_DIRECT>(M, T, slots, A, s);
@@ -1389,7 +1381,7 @@ cudaError_t slice_multi_launch(const Desc *D, const int2 *map, int nblocks, int 
 // Explicit instantiation of the launchers of one (precision, detectors) pair.
 #define GWNS_INSTANTIATE(P, D)                                                                       \
     template int slice_ws_blocks_per_sm<P, D>();                                                     \
-    template cudaError_t eval_launch<P, D>(const Model &, const Tables &, int, const double *, int, int, \
+    template cudaError_t eval_launch<P, D>(const Model &, const Tables &, int, int, const double *, int, int, \
                                            double *, RunState *, cudaStream_t);                     \
     template cudaError_t slice_launch<P, D>(const Model &, const Tables &, int, const StepArgs &,     \
                                             cudaStream_t);                                          \
