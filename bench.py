@@ -51,9 +51,6 @@ REF_STEPS = 2
 CLOCK_QUERY = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,"
                "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
                "clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
-# FP64 pipe peak derived from the unit count: 2 FP64 FMA per clock per SM
-# (1.25 TFLOP/s nominal over 152 SMs at 2070 MHz).
-FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 FP32_LANE_OPS = 152 * 128 * 2.070e9    # FP32 pipe: 128 lanes/clk/SM x 152 SMs x 2070 MHz
 SFU_LANE_OPS = 152 * 16 * 2.070e9      # MUFU (sin, cos): 16 lanes/clk/SM x 152 SMs x 2070 MHz
@@ -93,16 +90,6 @@ def recorded_traffic():
     if not (m_sha and m_b) or m_sha.group(1) != kernel_source_sha16():
         return None, None
     return int(m_b.group(1)), (int(m_pb.group(1)) if m_pb else None)
-
-
-def fp64_flops_per_point_bin(n_det: int) -> float:
-    """FP64 work of one point-bin summed bin by bin in FP64 instructions, in flops
-    (2 per FMA-equivalent): the phase as 8 basis FMAs, one sine/cosine pair (32
-    FMA-equivalents), and per detector the complex product with the weighted
-    data and one Horner step of a detector rotation (8). The FP64 form takes
-    neither these instructions nor, on long grids, every bin: its rate in these
-    units says what the FP64 pipe would have to reach."""
-    return 2.0 * (8 + 32 + 8 * n_det)
 
 
 def world():
@@ -397,9 +384,9 @@ def fp64_first_iteration(g, w, inputs, stream, flush):
     sp.close()
     t = sum(ms) / 1e3
     return {"evals_per_s": ev / t, "ms_per_step": sum(ms), "evals": ev, "point_bins_per_s": pb / t,
-            "k_slice_fp64_pipe_equivalent": pb * fp64_flops_per_point_bin(w.n_det) / (kern[3] / 1e3) / (FP64_PEAK_TFLOPS * 1e12),
-            "note": "first iteration, one step, CUDA events; the equivalent is the FP64 instructions of a bin-by-bin "
-                    "sum over the FP64 pipe's derived peak (2 FMA/clk/SM): the form runs off that pipe"}
+            "k_slice_ms": kern[3],
+            "note": "first iteration, one step, CUDA events; point-bins are those below each evaluation's cutoff, "
+                    "most of which the form sums as node rows"}
 
 
 def per_point_agreement(g, w, inputs, stream, points=1024):
@@ -852,7 +839,6 @@ def batch_eval_row(g, name, precision, stream, points=2048, reps=3, warps=0):
            "batch_evals_per_s": points * reps / t, "point_bins_per_s": pb / t, "bins_per_eval": pb / (points * reps)}
     if precision == g.NS_FP64:
         row["frac"], row["pipe"] = None, None
-        row["fp64_pipe_equivalent"] = pb * fp64_flops_per_point_bin(w.n_det) / t / (FP64_PEAK_TFLOPS * 1e12)
     else:
         row["frac"], row["pipe"] = mixed_roofline(pb, t, w.n_det, st1["mixed_tile"])
         row["mixed_tile"] = st1["mixed_tile"]
@@ -891,10 +877,9 @@ def oracle_rate(name: str, chains: int, steps_per_dim: int, target_s: float):
 
 
 def run_table(args):
-    """One JSON line per (workload, form): full runs of c0, c1, c2 and c4 on
-    1024 coarse bins (FP64 and mixed), c4 on the full grid (mixed: the whole
-    run; FP64: one iteration, and the batched likelihood), and the oracle's rate
-    per workload."""
+    """One JSON line per (workload, form): full runs of c0, c1, c2, c4 on 1024
+    coarse bins and c4 on the full grid (FP64 and mixed), the batched likelihood on
+    c2 and c4, and the oracle's rate per workload."""
     import torch
     import paper_2509_24949_gb300 as g
     from paper_2509_24949_gb300 import _build
@@ -907,8 +892,7 @@ def run_table(args):
             rows.append(table_row(g, name, prec, stream))
     for prec in (g.NS_FP64, g.NS_MIXED):
         rows.append(table_row(g, "c4", prec, stream, coarse=True))
-    rows.append(table_row(g, "c4", g.NS_MIXED, stream))                  # the whole run (~17 s)
-    rows.append(table_row(g, "c4", g.NS_FP64, stream, max_steps=1))      # one iteration
+        rows.append(table_row(g, "c4", prec, stream))
     for name in ("c2", "c4"):
         rows.append(batch_eval_row(g, name, g.NS_FP64, stream, points=2048))
         rows.append(batch_eval_row(g, name, g.NS_MIXED, stream, points=8192))
