@@ -210,19 +210,19 @@ DFI void fx_layout(const FxTiles &T, const FxBlocks *K, bool tiles, int n, FxPoi
 }
 DFI void fx_segments(const FxTiles &T, bool tiles, int n, FxPoint &o) { fx_layout(T, nullptr, tiles, n, o); }
 
-// The blocks of a grid. FP64 rounds a bin's phase by its size there, about the
-// Newtonian term 3/128 (pi T_sun Mc f)^(-5/3) (at the prior's lowest chirp mass mc)
-// plus 2 pi f tau (tau a typical delay) plus 10 rad for the rest; the split
-// arithmetic rounds it by the block's largest term at 2^-5 to 2^-6 of that. So a
+// The blocks of a grid. FP64 rounds a bin's phase by its size there: the Newtonian
+// term 3/128 (pi T_sun Mc f)^(-5/3) (at the prior's lowest chirp mass mc), twice
+// 2 pi f tau (tau a typical delay: its product and its sum are rounded) and 20 rad
+// for the rest; the split arithmetic rounds it by the block's largest term at 2^-5 to 2^-6 of that. So a
 // block ends where the phases have fallen to 1/40 of its first bin's Newtonian term
 // (a larger fall only where FX_BLK blocks do not suffice, on more than five decades of
-// frequency). From 20 Hz, chirp masses of 10 or more take one block, of 1.1 or more two.
+// frequency). From 20 Hz, chirp masses of 1.1 or more take one block.
 // A block's largest values are taken over its bins and the tiles that start in it,
 // whose nodes reach half a bin beyond the tile's bins. Every basis function is
 // monotone between its ends but f^(1/3) ln f, whose minimum is -3/e at f = e^-3.
 inline void fx_make_blocks(int N, double f0, double df, double mc, double tau, const FxTiles &T, FxBlocks &K) {
     const double f1 = f0 + (double)(N - 1) * df;
-    auto newton = [&](double f) { return 3.0 / 128.0 * pow(3.141592653589793 * 4.925490947641267e-6 * mc * f, -5.0 / 3.0); };
+    auto newton = [&](double f) { return 0.0234375 * pow(3.141592653589793 * 4.925490947641267e-6 * mc * f, -5.0 / 3.0); };
     double fall = 40.0;
     for (int it = 0; it < 64; it++, fall *= 1.5) {
         K.n = 1;
@@ -230,7 +230,7 @@ inline void fx_make_blocks(int N, double f0, double df, double mc, double tau, c
         int more = 0;
         double top = newton(f0);
         for (double f = f0; f < f1; f *= 1.09) {
-            if (!(top > fall * (newton(f) + 6.283185307179586 * f * tau + 10.0))) continue;
+            if (!(top > fall * (newton(f) + 12.566370614359172 * f * tau + 20.0))) continue;
             const double j = ceil((f - f0) / df);
             if (!(j < (double)N)) break;
             top = newton(f);

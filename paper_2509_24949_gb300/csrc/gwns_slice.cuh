@@ -299,9 +299,13 @@ __global__ void __launch_bounds__(W * 32, BLOCKS) k_eval_batch(Model M, Tables T
 constexpr int EVAL_FX_W = 4;                // warps
 constexpr int EVAL_FX_P = EVAL_FX_W;        // points at most
 
-// Relative binning (RB): one warp sums a point's coarse bins (C = 1).
+// Relative binning (RB): one warp sums a point's coarse bins (C = 1). Four CTAs an
+// SM; three for four detectors' rows, whose arithmetic wants more registers (64 / 1000
+// draws of 519,169 bins 112 / 407 -> 103 / 385 us; coarse bins 297 -> 317 us of 8192, so not
+// there).
+#define EVAL_FX_BLOCKS(NDET, RB) ((NDET) == 4 && !(RB) ? 3 : 16 / EVAL_FX_W)
 template <int NDET, bool RB>
-__global__ void __launch_bounds__(EVAL_FX_W * 32, 16 / EVAL_FX_W) k_eval_fx(Model M, Tables T, const double *in,
+__global__ void __launch_bounds__(EVAL_FX_W * 32, EVAL_FX_BLOCKS(NDET, RB)) k_eval_fx(Model M, Tables T, const double *in,
                                                                             int m, int P, int C, double *logl,
                                                                             RunState *st) {
     __shared__ Coef coef[EVAL_FX_P];

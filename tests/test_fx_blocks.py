@@ -241,10 +241,10 @@ def test_sums_against_fp64(fx, f1, N, masses, points):
 
 
 @pytest.mark.parametrize("N,f0,df,mc,tau,first,blocks", [
-    (9000, 20.0, 0.25, 10.0, 0.06, [], 1), (9000, 20.0, 0.25, 1.1, 0.06, [0], 2), (9000, 3.0, 0.25, 1.1, 0.06, [64, 256], 3),
+    (9000, 20.0, 0.25, 10.0, 0.06, [], 1), (9000, 20.0, 0.25, 1.1, 0.06, [0], 1), (9000, 3.0, 0.25, 1.1, 0.06, [64, 256], 2),
     (70000, 20.0, 1 / 32, 1.1, 0.0, [192, 256, 512, 1024, 2048], 2), (1, 20.0, 1.0, 1.1, 0.06, [], 1), (2, 0.01, 100.0, 1.1, 0.06, [], 2),
-    (5000, 0.01, 0.5, 1.1, 0.06, [], 6), (300, 1e-4, 10.0, 1.1, 0.06, [], 3), (3000000, 1e-6, 1e-4, 1.1, 0.06, [], 6),
-    (40, 5.0, 1e-3, 1.1, 0.06, [], 1), (3000, 0.01, 1.0, 1e-4, 0.0, [], 6)])
+    (5000, 0.01, 0.5, 1.1, 0.06, [], 5), (300, 1e-4, 10.0, 1.1, 0.06, [], 3), (3000000, 1e-6, 1e-4, 1.1, 0.06, [], 6),
+    (40, 5.0, 1e-3, 1.1, 0.06, [], 1), (3000, 0.01, 1.0, 1e-4, 0.0, [], 5)])
 def test_blocks_cover_the_grid(fx, N, f0, df, mc, tau, first, blocks):
     """Blocks start at bin 0 and ascend; every bin's and node's basis values stay below their block's
     power of two; a point's rows change block at the first bin, or the first tile, that starts in the next."""
