@@ -67,7 +67,7 @@ enum { NS_KERNEL_SLICE = 0, NS_KERNEL_WALK = 1 };
  * over bins are no further from the exact ones than FP64 instructions make them;
  * long grids are summed over the nodes of tiles, which makes this the faster form on
  * the longest: a GB300 runs an analysis of 519,169 bins in 7.2 s, mixed in 12.4 s;
- * 64,897 bins 0.79 s against 0.53 s).
+ * 64,897 bins 0.80 s against 0.54 s).
  * NS_MIXED: per-point coefficients in double-float (pairs of floats on the FP32
  * pipe; the FP64 stage instead when the environment variable GWNS_COEF_FP64=1 is
  * set at ns_init, or for relative binning), the per-bin phase in double-float,
