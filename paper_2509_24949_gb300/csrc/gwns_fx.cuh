@@ -10,9 +10,9 @@
 //    to their largest value there, a point's coefficients 60-bit integers on one
 //    scale per point and block: the unit is 2^-59 of the power of two above the
 //    point's largest term in the block, where FP64 rounds that term at 2^-53, so
-//    that also a block's last bins are rounded below FP64's sums (0.01 to 0.5 of their rms,
-//    by octave). One scale for a whole grid would give every bin the rounding of
-//    the lowest frequency's terms: rms error of the phases at 50 to 400 Hz, chirp
+//    that also a block's last bins are rounded below FP64's sums (0.01 to 0.5 of
+//    their rms, by octave). One scale for a whole grid would give every bin the
+//    rounding of the lowest frequency's terms: rms error of the phases at 50 to 400 Hz, chirp
 //    mass 1.2, grid from 20 / 5 / 1 / 0.1 Hz, FP64 1.3e-13 rad, one scale with
 //    58-bit coefficients and floored halves 5e-13 / 7e-12 / 1.2e-10 / 3.9e-9, blocks
 //    1.0e-13 (the tabulated basis' own rounding).
@@ -213,10 +213,11 @@ DFI void fx_segments(const FxTiles &T, bool tiles, int n, FxPoint &o) { fx_layou
 // The blocks of a grid. FP64 rounds a bin's phase by its size there: the Newtonian
 // term 3/128 (pi T_sun Mc f)^(-5/3) (at the prior's lowest chirp mass mc), twice
 // 2 pi f tau (tau a typical delay: its product and its sum are rounded) and 20 rad
-// for the rest; the split arithmetic rounds it by the block's largest term at 2^-5 to 2^-6 of that. So a
-// block ends where the phases have fallen to 1/40 of its first bin's Newtonian term
-// (a larger fall only where FX_BLK blocks do not suffice, on more than five decades of
-// frequency). From 20 Hz, chirp masses of 1.1 or more take one block.
+// for the rest; the split arithmetic rounds it by the block's largest term at 2^-5
+// to 2^-6 of that. So a block ends where the phases have fallen to 1/40 of its first
+// bin's Newtonian term (a larger fall only where FX_BLK blocks do not suffice, on
+// more than five decades of frequency). From 20 Hz, chirp masses of 1.1 or more take
+// one block.
 // A block's largest values are taken over its bins and the tiles that start in it,
 // whose nodes reach half a bin beyond the tile's bins. Every basis function is
 // monotone between its ends but f^(1/3) ln f, whose minimum is -3/e at f = e^-3.
@@ -229,7 +230,8 @@ inline void fx_make_blocks(int N, double f0, double df, double mc, double tau, c
         K.bin[0] = 0;
         int more = 0;
         double top = newton(f0);
-        for (double f = f0; f < f1; f *= 1.09) {
+        double f = f0;
+        for (int s = 0; s < (1 << 14) && f < f1; s++, f *= 1.09) {      // (a subnormal f may not grow)
             if (!(top > fall * (newton(f) + 12.566370614359172 * f * tau + 20.0))) continue;
             const double j = ceil((f - f0) / df);
             if (!(j < (double)N)) break;
@@ -258,7 +260,7 @@ inline void fx_make_blocks(int N, double f0, double df, double mc, double tau, c
             for (int m = 0; m <= FX_NB; m++) mx[m] = fmax(mx[m], fabs(B[m]));
         }
         if (lo < 0.05 && hi > 0.049) mx[6] = fmax(mx[6], 1.2);
-        for (int m = 0; m <= FX_NB; m++) K.e[b][m] = ilogb(fmax(mx[m] * (1.0 + 1e-12), 1e-300)) + 1;
+        for (int m = 0; m <= FX_NB; m++) K.e[b][m] = ilogb(fmin(fmax(mx[m] * (1.0 + 1e-12), 1e-300), 1e300)) + 1;
     }
 }
 

@@ -240,6 +240,17 @@ def test_sums_against_fp64(fx, f1, N, masses, points):
     assert split <= 1.05 * fp64, (split, fp64)
 
 
+@pytest.mark.parametrize("f0", [5e-324, 1e-310, 1e-200, 1e-60])
+def test_blocks_of_the_smallest_frequencies(fx, f0):
+    """Grids that start where the basis functions overflow are accepted too: the rule ends, with blocks
+    that ascend from bin 0 and exponents of a double."""
+    out = list(map(int, fx([f"b 300 {f0!r} 10.0 1.1 0.06 0 1 300"])[0].split()))
+    nb = out[0]
+    bins, e = [out[1 + 10 * b] for b in range(nb)], [out[2 + 10 * b:11 + 10 * b] for b in range(nb)]
+    assert 1 <= nb <= 6 and bins[0] == 0 and all(a < b < 300 for a, b in zip(bins, bins[1:]))
+    assert all(abs(k) <= 1074 for v in e for k in v)
+
+
 @pytest.mark.parametrize("N,f0,df,mc,tau,first,blocks", [
     (9000, 20.0, 0.25, 10.0, 0.06, [], 1), (9000, 20.0, 0.25, 1.1, 0.06, [0], 1), (9000, 3.0, 0.25, 1.1, 0.06, [64, 256], 2),
     (70000, 20.0, 1 / 32, 1.1, 0.0, [192, 256, 512, 1024, 2048], 2), (1, 20.0, 1.0, 1.1, 0.06, [], 1), (2, 0.01, 100.0, 1.1, 0.06, [], 2),
